@@ -96,7 +96,9 @@ enum {
                                    else, at r in {4, 8}, the narrow-tile FMA pass when its
                                    tiles number at most half of the 32-row tiles (sets of
                                    thin matrices such as LoRA factors); else the FMA pass,
-                               1 = FMA path on 32-row tiles, 2 = tcgen05 path,
+                               1 = FMA path on full tiles (64 x 128; at r in {4, 8} and at
+                               most four waves of them one-launch passes on 32-row tiles),
+                               2 = tcgen05 path,
                                3 = FMA path on narrow tiles (r in {4, 8}).  All FMA
                                tilings give bit-identical weights. */
   ZO_OPTION_TIMING = 1,     /* 1 = record CUDA events around every weight-pass launch */
@@ -272,7 +274,7 @@ ZO_API zo_status zo_set_option(zo_ctx* ctx, int32_t option, int64_t value);
 ZO_API zo_status zo_get_timing(zo_ctx* ctx, double* total_ms, int64_t* launches);
 
 /* zo_wpass_path -- the weight-pass path the last zo_perturb / zo_step launched
-   (1 = FMA on 32-row tiles, 2 = tcgen05, 3 = FMA on narrow tiles). */
+   (1 = FMA on full tiles, 2 = tcgen05, 3 = FMA on narrow tiles). */
 ZO_API int32_t zo_wpass_path(const zo_ctx* ctx);
 
 /* zo_linear_tiling -- the tiling (1 .. 8, as ZO_OPTION_LINEAR_TILE) of the Y GEMM that

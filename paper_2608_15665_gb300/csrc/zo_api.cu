@@ -76,6 +76,9 @@ struct zo_ctx {
   zo::MatDesc* d_mats = nullptr;
   int64_t* d_tile_prefix = nullptr;
   int64_t n_tiles = 0;
+  // the FMA pass from P: its tiles
+  int64_t* d_gemm_prefix = nullptr;
+  int64_t n_gemm_tiles = 0;
   // narrow tiles of the FMA path (r in {4, 8}); chosen automatically when they need at
   // most half the CTAs of the 32-row tiles
   zo::NarrowMat* d_narrow = nullptr;
@@ -167,6 +170,7 @@ void free_ctx(zo_ctx* c) {
   if (!c) return;
   cudaFree(c->d_mats);
   cudaFree(c->d_tile_prefix);
+  cudaFree(c->d_gemm_prefix);
   cudaFree(c->d_narrow);
   cudaFree(c->d_narrow_tiles);
   cudaFree(c->d_proj_units);
@@ -349,8 +353,8 @@ zo_status run_weight_pass(zo_ctx* c) {
     }
     c->last_path = 2;
   } else {
-    ZO_CUDA(zo::launch_wpass_fma(c->d_mats, c->n_mats, c->d_tile_prefix, c->n_tiles, c->r,
-                                 c->stream),
+    ZO_CUDA(zo::launch_wpass_gemm(c->d_mats, c->n_mats, c->d_gemm_prefix, c->n_gemm_tiles,
+                                  c->r, c->stream),
             "weight-pass kernel");
     c->last_path = 1;
   }
@@ -646,7 +650,7 @@ zo_status zo_create(zo_ctx** out, const zo_matrix* mats, int32_t n_mats, int32_t
   }
 
   // weight-pass tiles and projection units
-  std::vector<int64_t> prefix(n_mats + 1, 0);
+  std::vector<int64_t> prefix(n_mats + 1, 0), gemm_prefix(n_mats + 1, 0);
   std::vector<int2> units;
   c->h_mats.resize(n_mats);
   for (int32_t i = 0; i < n_mats; ++i) {
@@ -668,10 +672,12 @@ zo_status zo_create(zo_ctx** out, const zo_matrix* mats, int32_t n_mats, int32_t
     const int64_t tiles = ((mt.m + zo::kFmaTileRows - 1) / zo::kFmaTileRows) * ((mt.n + tn - 1) / tn);
     d.tile0 = prefix[i];
     prefix[i + 1] = prefix[i] + tiles;
+    gemm_prefix[i + 1] = gemm_prefix[i] + zo::wpass_gemm_tiles(mt.m, mt.n);
     for (int64_t j0 = 0; j0 < mt.n; j0 += 128) units.push_back(make_int2(i, (int)j0));
     c->h_mats[i] = d;
   }
   c->n_tiles = prefix[n_mats];
+  c->n_gemm_tiles = gemm_prefix[n_mats];
   c->n_proj_units = (int32_t)units.size();
   if (c->n_tiles > 0x7FFFFFFF) {
     g_last_error = "too many weight-pass tiles";
@@ -731,6 +737,7 @@ zo_status zo_create(zo_ctx** out, const zo_matrix* mats, int32_t n_mats, int32_t
   e = cudaMalloc(&c->d_losses, sizeof(float) * c->max_losses);
   if (e == cudaSuccess) e = cudaMalloc(&c->d_mats, sizeof(zo::MatDesc) * n_mats);
   if (e == cudaSuccess) e = cudaMalloc(&c->d_tile_prefix, sizeof(int64_t) * (n_mats + 1));
+  if (e == cudaSuccess) e = cudaMalloc(&c->d_gemm_prefix, sizeof(int64_t) * (n_mats + 1));
   if (e == cudaSuccess) e = cudaMalloc(&c->d_proj_units, sizeof(int2) * std::max<size_t>(units.size(), 1));
   if (e == cudaSuccess) e = cudaMalloc(&c->d_qr_blocks, sizeof(zo::QrBlock) * std::max<size_t>(all_blocks.size(), 1));
   if (e == cudaSuccess) e = cudaMalloc(&c->d_status, sizeof(uint32_t));
@@ -749,6 +756,8 @@ zo_status zo_create(zo_ctx** out, const zo_matrix* mats, int32_t n_mats, int32_t
   e = cudaMemcpy(c->d_mats, c->h_mats.data(), sizeof(zo::MatDesc) * n_mats, cudaMemcpyHostToDevice);
   if (e == cudaSuccess)
     e = cudaMemcpy(c->d_tile_prefix, prefix.data(), sizeof(int64_t) * (n_mats + 1), cudaMemcpyHostToDevice);
+  if (e == cudaSuccess)
+    e = cudaMemcpy(c->d_gemm_prefix, gemm_prefix.data(), sizeof(int64_t) * (n_mats + 1), cudaMemcpyHostToDevice);
   if (e == cudaSuccess && !units.empty())
     e = cudaMemcpy(c->d_proj_units, units.data(), sizeof(int2) * units.size(), cudaMemcpyHostToDevice);
   if (e == cudaSuccess && !all_blocks.empty())

@@ -22,6 +22,17 @@ enum DeviceStatus : uint32_t {
   kDevNotPosDef = 4, // refresh: a Gram matrix had a non-positive Cholesky pivot
 };
 
+// Two fp32 multiply-adds (each rounded once, as fmaf) in one instruction.
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {
+  float2 d;
+  asm("{\n\t.reg .b64 a, b, c, d;\n\t"
+      "mov.b64 a, {%2, %3};\n\tmov.b64 b, {%4, %5};\n\tmov.b64 c, {%6, %7};\n\t"
+      "fma.rn.f32x2 d, a, b, c;\n\tmov.b64 {%0, %1}, d;\n\t}"
+      : "=f"(d.x), "=f"(d.y)
+      : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y), "f"(c.x), "f"(c.y));
+  return d;
+}
+
 // ---------------------------------------------------------------------------
 // Counter contract
 // ---------------------------------------------------------------------------
@@ -91,7 +102,7 @@ struct MatDesc {
   float* Vm;        // r x r second moment
   float* C;         // r x r coefficient of the current pass (workspace)
   float* P;         // FMA path: r x n, P = C V^T (workspace)
-  int64_t tile0;    // first weight-pass tile of this matrix (FMA path)
+  int64_t tile0;    // first 32-row tile of this matrix (one-launch FMA passes, MeZO)
 };
 
 // Per-matrix record of the tensor-core weight pass (128 x 128 tiles).

@@ -53,12 +53,17 @@ cudaError_t launch_project_fma(const MatDesc* d_mats, const int2* d_units, int32
                                int32_t r, cudaStream_t s);
 
 
-// ---- weight pass, fp32 FMA path (zo_wpass_fma.cu) ---------------------------
+// ---- weight pass, fp32 FMA path (zo_wpass_gemm.cu, zo_wpass_fma.cu) -----------------
+// From P, on 64 x 128 tiles: matrix i's from d_prefix[i] on (n_mats + 1 entries).
+constexpr int kGemmTileRows = 64;
+constexpr int kGemmTileCols = 128;
+int64_t wpass_gemm_tiles(int64_t m, int64_t n);
+cudaError_t launch_wpass_gemm(const MatDesc* d_mats, int32_t n_mats, const int64_t* d_prefix,
+                              int64_t n_tiles, int32_t r, cudaStream_t s);
+
+// The 32-row tiles of the one-launch passes (d_tile_prefix, MatDesc::tile0).
 constexpr int kFmaTileRows = 32;
 __host__ __device__ constexpr int fma_tile_cols(int32_t dtype) { return dtype == 1 ? 256 : 128; }
-
-cudaError_t launch_wpass_fma(const MatDesc* d_mats, int32_t n_mats, const int64_t* d_tile_prefix,
-                             int64_t n_tiles, int32_t r, cudaStream_t s);
 
 // One-launch perturbation pass of the FMA path at r in {4, 8}: each CTA forms C from p
 // (mode kCoeffPerturb) and its tile's P columns itself (zo_wpass_fma.cu).

@@ -9,10 +9,12 @@
 // (integer multiplies, log / sqrt / sincos), not by HBM.  Tiles are the FMA pass's
 // 32 rows x (32 lanes x 16 bytes): a warp reads and writes 512 contiguous bytes of
 // a row, each thread draws the 2 (bf16) or 1 (fp32) counter words of its 16 bytes.
-#include "zo_kernels.h"
+#include "zo_fma_common.cuh"
 
 namespace zo {
 namespace {
+
+using namespace fma;
 
 constexpr uint32_t kTagMezo = 5;
 
@@ -53,26 +55,11 @@ __device__ __forceinline__ float4 normal4_keyed(const RoundKeys& k, uint32_t c4,
   return make_float4(a.x, a.y, b.x, b.y);
 }
 
-__device__ __forceinline__ int find_matrix_tile(const int64_t* __restrict__ prefix, int n_mats,
-                                                int64_t tile) {
-  int lo = 0, hi = n_mats - 1;
-  while (lo < hi) {
-    const int mid = (lo + hi + 1) >> 1;
-    if (__ldg(prefix + mid) <= tile) lo = mid; else hi = mid - 1;
-  }
-  return lo;
-}
-
-__device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
-  const __nv_bfloat162 h = __floats2bfloat162_rn(lo, hi);
-  return *reinterpret_cast<const uint32_t*>(&h);
-}
-
 __global__ void __launch_bounds__(256)
 mezo_kernel(const MatDesc* __restrict__ mats, int n_mats, const int64_t* __restrict__ prefix,
             const __grid_constant__ RoundKeys keys, uint32_t t, float coef) {
   const int64_t tile = blockIdx.x;
-  const MatDesc md = mats[find_matrix_tile(prefix, n_mats, tile)];
+  const MatDesc md = mats[find_matrix(prefix, n_mats, tile)];
   const int bf16 = md.dtype == 1;
   const int vec = bf16 ? 8 : 4;                       // elements per 16 bytes
   const int64_t tn = 32 * vec;                        // tile columns
@@ -105,7 +92,7 @@ mezo_kernel(const MatDesc* __restrict__ mats, int n_mats, const int64_t* __restr
         for (int k = 0; k < 4; ++k) {
           const float lo = fmaf(coef, z[2 * k], __uint_as_float(v[k] << 16));
           const float hi = fmaf(coef, z[2 * k + 1], __uint_as_float(v[k] & 0xFFFF0000u));
-          o[k] = pack_bf16x2(lo, hi);
+          o[k] = pack2_bf16(lo, hi);
         }
         *reinterpret_cast<uint4*>(w) = make_uint4(o[0], o[1], o[2], o[3]);
       } else {

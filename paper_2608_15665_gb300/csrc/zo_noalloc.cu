@@ -94,8 +94,7 @@ extern "C" ZO_API zo_status zo_perturb_noalloc(void* W, int64_t m, int64_t n, in
     return fail(ZO_ERR_SHAPE, "zo_perturb_noalloc needs " + std::to_string(L.total) +
                                   " floats of scratch (r*n + r*r + tables); its static scratch holds " +
                                   std::to_string(kScratchFloats) + " floats (8 MiB)");
-  const int64_t tiles = ((m + zo::kFmaTileRows - 1) / zo::kFmaTileRows) *
-                        ((n + zo::fma_tile_cols(dtype) - 1) / zo::fma_tile_cols(dtype));
+  const int64_t tiles = zo::wpass_gemm_tiles(m, n);
   if (tiles > 0x7FFFFFFF) return fail(ZO_ERR_SHAPE, "too many weight-pass tiles");
 
   int dev = 0;
@@ -160,7 +159,7 @@ extern "C" ZO_API zo_status zo_perturb_noalloc(void* W, int64_t m, int64_t n, in
   p.eps = eps;
   e = zo::launch_coeff(d_desc, 1, p, s);
   if (e == cudaSuccess) e = zo::launch_project_fma(d_desc, d_units, (int32_t)n_units, r, s);
-  if (e == cudaSuccess) e = zo::launch_wpass_fma(d_desc, 1, d_prefix, tiles, r, s);
+  if (e == cudaSuccess) e = zo::launch_wpass_gemm(d_desc, 1, d_prefix, tiles, r, s);
   if (e != cudaSuccess) return fail(ZO_ERR_CUDA, std::string("launch: ") + cudaGetErrorString(e));
   return ZO_OK;
 }

@@ -1,27 +1,26 @@
-// Weight pass, fp32-FMA path: W_i <- rnd(W_i + U_i P_i) for every matrix in one
-// launch, with P_i = C_i V_i^T precomputed (r x n fp32).  This is the fused
-// form of Alg. 2's "W_i <- W_i + eps U_i Z_i V_i^T" (Eq. (4)) and of the update
-// of Eq. (10): the r-term contraction is done in fp32 FMAs and W is rounded once.
+// Weight pass, fp32-FMA path, one launch per perturbation pass at r in {4, 8}: each CTA
+// forms C_i and its tile's columns of P_i = C_i V_i^T itself and updates
+// W_i <- rnd(W_i + U_i P_i) -- the fused form of Alg. 2's "W_i <- W_i + eps U_i Z_i V_i^T"
+// (Eq. (4)).  The r-term contraction is done in fp32 FMAs and W is rounded once.  For sets
+// whose pass is bound by launches and latency; larger ones, and higher ranks, run
+// zo_wpass_gemm.cu.
 //
-// Tiling: a CTA owns a 32-row x TN-column tile of one W_i (TN = 32 lanes x 16 B).
-// Each thread keeps a 4-row x (16 B of W) register tile; W is read and written
-// with 16-byte coalesced vector accesses (a warp covers 512 contiguous bytes of
-// a row), U and P tiles are staged through shared memory.  HBM traffic per
-// element is one read and one write of W; U and P tiles come from L2.
+// Tiling: a CTA owns a 32-row x TN-column tile of one W_i (TN = 32 lanes x 16 B), or a
+// narrow tile shaped after its matrix (below).  Each thread keeps a 4-row x (16 B of W)
+// register tile; W is read and written with 16-byte coalesced vector accesses (a warp
+// covers 512 contiguous bytes of a row), U and P tiles sit in shared memory.
 #include <algorithm>
 #include <atomic>
 
-#include "zo_kernels.h"
+#include "zo_fma_common.cuh"
 
 namespace zo {
 namespace {
 
+using namespace fma;
+
 constexpr int kRows = kFmaTileRows;   // 32
 constexpr int kRowsPerThread = kRows / 8;   // 8 warps stacked over the tile rows
-
-template <typename T> struct Vec;
-template <> struct Vec<float> { static constexpr int N = 4; };
-template <> struct Vec<__nv_bfloat16> { static constexpr int N = 8; };
 
 __device__ __forceinline__ void unpack(const uint4& raw, float (&w)[4], float) {
   w[0] = __uint_as_float(raw.x); w[1] = __uint_as_float(raw.y);
@@ -39,46 +38,14 @@ __device__ __forceinline__ void unpack(const uint4& raw, float (&w)[8], __nv_bfl
     w[2 * i + 1] = __uint_as_float(v[i] & 0xFFFF0000u);
   }
 }
-__device__ __forceinline__ uint32_t pack2_bf16(float lo, float hi) {
-  const __nv_bfloat162 h = __floats2bfloat162_rn(lo, hi);   // RNE, lo in the low half
-  return *reinterpret_cast<const uint32_t*>(&h);
-}
 __device__ __forceinline__ uint4 pack(const float (&w)[8], __nv_bfloat16) {
   return make_uint4(pack2_bf16(w[0], w[1]), pack2_bf16(w[2], w[3]), pack2_bf16(w[4], w[5]),
                     pack2_bf16(w[6], w[7]));
 }
 
-template <typename T>
-__device__ __forceinline__ float load_scalar(const T* p);
-template <>
-__device__ __forceinline__ float load_scalar<float>(const float* p) { return *p; }
-template <>
-__device__ __forceinline__ float load_scalar<__nv_bfloat16>(const __nv_bfloat16* p) {
-  return __bfloat162float(*p);
-}
-template <typename T>
-__device__ __forceinline__ void store_scalar(T* p, float x);
-template <>
-__device__ __forceinline__ void store_scalar<float>(float* p, float x) { *p = x; }
-template <>
-__device__ __forceinline__ void store_scalar<__nv_bfloat16>(__nv_bfloat16* p, float x) {
-  *p = __float2bfloat16_rn(x);
-}
-
-__device__ __forceinline__ int find_matrix(const int64_t* __restrict__ prefix, int n_mats,
-                                           int64_t tile) {
-  int lo = 0, hi = n_mats - 1;
-  while (lo < hi) {
-    const int mid = (lo + hi + 1) >> 1;
-    if (__ldg(prefix + mid) <= tile) lo = mid; else hi = mid - 1;
-  }
-  return lo;
-}
-
-// With kFused, P's columns of this tile are formed here from C (already in shared memory,
-// Cs) and V, in the projection kernel's order (sum over b ascending, one fmaf per term),
-// instead of being read from md.P.
-template <int R, typename T, bool kFused>
+// P's columns of this tile are formed here from C (already in shared memory, Cs) and V, in
+// the projection kernel's order (sum over b ascending, one fmaf per term).
+template <int R, typename T>
 __device__ __forceinline__ void wpass_tile(const MatDesc& md, int64_t local, float* Us, float* Ps,
                                            const float* Cs) {
   constexpr int VEC = Vec<T>::N;
@@ -111,28 +78,18 @@ __device__ __forceinline__ void wpass_tile(const MatDesc& md, int64_t local, flo
       Us4[idx] = row < md.m ? U4[row0 * (R / 4) + idx] : make_float4(0.f, 0.f, 0.f, 0.f);
     }
     // layout [k][c % VEC / 4][c / VEC][c % 4]: a thread's 16-B chunks are contiguous across lanes
-    if constexpr (kFused) {
-      for (int c = tid; c < TN; c += blockDim.x) {
-        const int64_t gc = col0 + c;
-        const int lane = c / VEC, part = (c % VEC) / 4, l4 = c % 4;
-        float v[R];
+    for (int c = tid; c < TN; c += blockDim.x) {
+      const int64_t gc = col0 + c;
+      const int lane = c / VEC, part = (c % VEC) / 4, l4 = c % 4;
+      float v[R];
 #pragma unroll
-        for (int b = 0; b < R; ++b) v[b] = gc < md.n ? md.V[gc * R + b] : 0.f;
+      for (int b = 0; b < R; ++b) v[b] = gc < md.n ? md.V[gc * R + b] : 0.f;
 #pragma unroll
-        for (int k = 0; k < R; ++k) {
-          float acc = 0.f;
+      for (int k = 0; k < R; ++k) {
+        float acc = 0.f;
 #pragma unroll
-          for (int b = 0; b < R; ++b) acc = fmaf(Cs[k * R + b], v[b], acc);
-          Ps[k * TN + part * 128 + lane * 4 + l4] = gc < md.n ? acc : 0.f;
-        }
-      }
-    } else {
-      for (int idx = tid; idx < R * TN; idx += blockDim.x) {
-        const int k = idx / TN, c = idx % TN;
-        const int64_t gc = col0 + c;
-        const float pv = gc < md.n ? md.P[(int64_t)k * md.n + gc] : 0.f;
-        const int lane = c / VEC, part = (c % VEC) / 4, l4 = c % 4;
-        Ps[k * TN + part * 128 + lane * 4 + l4] = pv;
+        for (int b = 0; b < R; ++b) acc = fmaf(Cs[k * R + b], v[b], acc);
+        Ps[k * TN + part * 128 + lane * 4 + l4] = gc < md.n ? acc : 0.f;
       }
     }
   }
@@ -189,22 +146,6 @@ __device__ __forceinline__ void wpass_tile(const MatDesc& md, int64_t local, flo
   }
 }
 
-template <int R>
-__global__ void __launch_bounds__(256, 2)
-wpass_fma_kernel(const MatDesc* __restrict__ mats, int n_mats, const int64_t* __restrict__ prefix) {
-  extern __shared__ float4 smem4[];
-  float* Us = reinterpret_cast<float*>(smem4);
-  float* Ps = Us + kRows * R;
-  const int64_t tile = blockIdx.x;
-  const int i = find_matrix(prefix, n_mats, tile);
-  const MatDesc md = mats[i];
-  const int64_t local = tile - md.tile0;
-  if (md.dtype == 1)
-    wpass_tile<R, __nv_bfloat16, false>(md, local, Us, Ps, nullptr);
-  else
-    wpass_tile<R, float, false>(md, local, Us, Ps, nullptr);
-}
-
 // C = eps (ca Z_qa + cb Z_qb) of one matrix into shared memory, with the coefficient
 // kernel's arithmetic (so that every path forms the same C).
 template <int R>
@@ -241,9 +182,9 @@ wpass_fma_fused_kernel(const MatDesc* __restrict__ mats, int n_mats,
   __syncthreads();
   const int64_t local = tile - md.tile0;
   if (md.dtype == 1)
-    wpass_tile<R, __nv_bfloat16, true>(md, local, Us, Ps, Cs);
+    wpass_tile<R, __nv_bfloat16>(md, local, Us, Ps, Cs);
   else
-    wpass_tile<R, float, true>(md, local, Us, Ps, Cs);
+    wpass_tile<R, float>(md, local, Us, Ps, Cs);
 }
 
 // The dynamic shared-memory limit of a kernel belongs to each device's context: raise it
@@ -258,17 +199,6 @@ cudaError_t allow_smem(Kernel kernel, int bytes, std::atomic<uint64_t>& done) {
   e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
   if (e == cudaSuccess) done.fetch_or(bit, std::memory_order_relaxed);
   return e;
-}
-
-template <int R>
-cudaError_t launch_r(const MatDesc* d_mats, int32_t n_mats, const int64_t* d_prefix,
-                     int64_t n_tiles, cudaStream_t s) {
-  const size_t smem = sizeof(float) * (size_t)(kRows * R + R * 256);
-  static std::atomic<uint64_t> done{0};
-  cudaError_t e = allow_smem(wpass_fma_kernel<R>, (int)smem, done);
-  if (e != cudaSuccess) return e;
-  wpass_fma_kernel<R><<<(unsigned)n_tiles, 256, smem, s>>>(d_mats, n_mats, d_prefix);
-  return cudaGetLastError();
 }
 
 template <int R>
@@ -515,21 +445,6 @@ cudaError_t launch_wpass_narrow(const MatDesc* d_mats, const NarrowMat* d_narrow
     case 8:
       return draw ? launch_narrow_r<8, true>(d_mats, d_narrow, d_tiles, n_tiles, p, p_floats, u_floats, s)
                   : launch_narrow_r<8, false>(d_mats, d_narrow, d_tiles, n_tiles, p, p_floats, u_floats, s);
-    default: return cudaErrorInvalidValue;
-  }
-}
-
-cudaError_t launch_wpass_fma(const MatDesc* d_mats, int32_t n_mats, const int64_t* d_tile_prefix,
-                             int64_t n_tiles, int32_t r, cudaStream_t s) {
-  if (n_tiles <= 0) return cudaSuccess;
-  if (n_tiles > 0x7FFFFFFF) return cudaErrorInvalidValue;
-  switch (r) {
-    case 4: return launch_r<4>(d_mats, n_mats, d_tile_prefix, n_tiles, s);
-    case 8: return launch_r<8>(d_mats, n_mats, d_tile_prefix, n_tiles, s);
-    case 16: return launch_r<16>(d_mats, n_mats, d_tile_prefix, n_tiles, s);
-    case 32: return launch_r<32>(d_mats, n_mats, d_tile_prefix, n_tiles, s);
-    case 64: return launch_r<64>(d_mats, n_mats, d_tile_prefix, n_tiles, s);
-    case 128: return launch_r<128>(d_mats, n_mats, d_tile_prefix, n_tiles, s);
     default: return cudaErrorInvalidValue;
   }
 }
