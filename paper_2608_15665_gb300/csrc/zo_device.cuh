@@ -22,7 +22,7 @@ enum DeviceStatus : uint32_t {
   kDevNotPosDef = 4, // refresh: a Gram matrix had a non-positive Cholesky pivot
 };
 
-// Two fp32 multiply-adds (each rounded once, as fmaf) in one instruction.
+// Two fp32 operations (each lane rounded to nearest, as fmaf, * and +) in one instruction.
 __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {
   float2 d;
   asm("{\n\t.reg .b64 a, b, c, d;\n\t"
@@ -30,6 +30,24 @@ __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {
       "fma.rn.f32x2 d, a, b, c;\n\tmov.b64 {%0, %1}, d;\n\t}"
       : "=f"(d.x), "=f"(d.y)
       : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y), "f"(c.x), "f"(c.y));
+  return d;
+}
+__device__ __forceinline__ float2 mul2(float2 a, float2 b) {
+  float2 d;
+  asm("{\n\t.reg .b64 a, b, d;\n\t"
+      "mov.b64 a, {%2, %3};\n\tmov.b64 b, {%4, %5};\n\t"
+      "mul.rn.f32x2 d, a, b;\n\tmov.b64 {%0, %1}, d;\n\t}"
+      : "=f"(d.x), "=f"(d.y)
+      : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+  return d;
+}
+__device__ __forceinline__ float2 add2(float2 a, float2 b) {
+  float2 d;
+  asm("{\n\t.reg .b64 a, b, d;\n\t"
+      "mov.b64 a, {%2, %3};\n\tmov.b64 b, {%4, %5};\n\t"
+      "add.rn.f32x2 d, a, b;\n\tmov.b64 {%0, %1}, d;\n\t}"
+      : "=f"(d.x), "=f"(d.y)
+      : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
   return d;
 }
 
@@ -54,28 +72,152 @@ __device__ __forceinline__ uint4 philox4x32_10(uint4 c, uint32_t k0, uint32_t k1
       k0 += 0x9E3779B9u;
       k1 += 0xBB67AE85u;
     }
-    const uint32_t hi_a = __umulhi(0xD2511F53u, c.x);
-    const uint32_t lo_a = 0xD2511F53u * c.x;
-    const uint32_t hi_b = __umulhi(0xCD9E8D57u, c.z);
-    const uint32_t lo_b = 0xCD9E8D57u * c.z;
+    const uint64_t a = (uint64_t)0xD2511F53u * c.x, b = (uint64_t)0xCD9E8D57u * c.z;
+    const uint32_t hi_a = (uint32_t)(a >> 32), lo_a = (uint32_t)a;
+    const uint32_t hi_b = (uint32_t)(b >> 32), lo_b = (uint32_t)b;
     c = make_uint4(hi_b ^ c.y ^ k0, lo_b, hi_a ^ c.w ^ k1, lo_a);
   }
   return c;
 }
 
-// u = ((x >> 8) + 1) * 2^-24 in (0, 1]; the integer fits 24 bits, so exact in fp32.
-__device__ __forceinline__ float u01(uint32_t x) {
-  return __uint2float_rn((x >> 8) + 1u) * 5.9604644775390625e-08f;
+// The transform below runs on one value at a time (float) or on packed pairs (float2); both
+// round every operation alike, so they give the same bits.
+__device__ __forceinline__ float vfma(float a, float b, float c) { return fmaf(a, b, c); }
+__device__ __forceinline__ float2 vfma(float2 a, float2 b, float2 c) { return fma2(a, b, c); }
+__device__ __forceinline__ float vmul(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ float2 vmul(float2 a, float2 b) { return mul2(a, b); }
+__device__ __forceinline__ float vadd(float a, float b) { return __fadd_rn(a, b); }
+__device__ __forceinline__ float2 vadd(float2 a, float2 b) { return add2(a, b); }
+template <typename V> struct Lanes;
+template <> struct Lanes<float> {
+  static constexpr int N = 1;
+  static __device__ __forceinline__ float all(float x) { return x; }
+  static __device__ __forceinline__ float from(const float* x) { return x[0]; }
+  static __device__ __forceinline__ void to(float v, float* x) { x[0] = v; }
+};
+template <> struct Lanes<float2> {
+  static constexpr int N = 2;
+  static __device__ __forceinline__ float2 all(float x) { return make_float2(x, x); }
+  static __device__ __forceinline__ float2 from(const float* x) { return make_float2(x[0], x[1]); }
+  static __device__ __forceinline__ void to(float2 v, float* x) { x[0] = v.x; x[1] = v.y; }
+};
+
+// Box-Muller on kV vectors of word pairs (xa, xb), u = ((x >> 8) + 1) 2^-24 in (0, 1]:
+// rad cos 2 pi ub = nr c and rad sin 2 pi ub = nr s with nr = -rad = -sqrt(-2 ln ua).  The
+// uniforms are integers over 2^24, so both functions reduce their arguments exactly, in
+// integers; the polynomials are minimax fits whose coefficients are rounded from the lowest
+// order on, the rest refitted:
+//  * ln: k = u 2^24 = m 2^e with m in [2/3, 4/3), g = 2 m - 2 exact, 2 ln u = (e - 24) 2 ln 2
+//    + g + g^2 P(g), P of degree 8 (5.0e-9 of the result).
+//  * sqrt of x = -2 ln u: the hardware's reciprocal square root y, s = x y, and one Newton
+//    step s + (x - s^2) y / 2, all with the sign turned; u = 1 gives 0.
+//  * cos, sin: k + 2^21 = quadrant 2^22 + j, the angle inside the quadrant (pi/4) t with
+//    t = (j - 2^21) 2^-21 exact in [-1, 1); sin = t s0 + t q(t^2) with s0 the fp32 pi/4 and
+//    its error in q, cos = 1 + t^2 p(t^2) (2.5e-9 and 6e-11); the quadrant swaps and negates.
+// Over all 2^24 uniforms (double precision): radius within 3.5e-7 (rms 4.05e-8), cos and sin
+// within 6.1e-8, no further off than logf, sqrtf and sincospif.
+template <int kV, typename V>
+__device__ __forceinline__ void box_muller_parts(const uint32_t (&xa)[kV * Lanes<V>::N],
+                                                 const uint32_t (&xb)[kV * Lanes<V>::N],
+                                                 V (&nr)[kV], V (&zc)[kV], V (&zs)[kV]) {
+  using LN = Lanes<V>;
+  constexpr int kL = LN::N, kN = kV * kL;
+  {
+    V g[kV], e[kV], P[kV];
+#pragma unroll
+    for (int v = 0; v < kV; ++v) {
+      float m[kL], x[kL];
+#pragma unroll
+      for (int l = 0; l < kL; ++l) {
+        const int k = __float_as_int(__uint2float_rn((xa[v * kL + l] >> 8) + 1u));
+        const int ex = (k - 0x4b2aaaab) & (int)0xff800000;     // (e - 24) 2^23
+        m[l] = __int_as_float(k - ex - 0x0c000000);
+        x[l] = __int2float_rn(ex);
+      }
+      g[v] = vfma(LN::from(m), LN::all(2.0f), LN::all(-2.0f));
+      e[v] = LN::from(x);
+    }
+    constexpr float kP[9] = {-0x1p-2f,        0x1.55550cp-4f,  -0x1.fffe5ep-6f,
+                             0x1.99ce34p-7f,  -0x1.55b7ecp-8f, 0x1.1ef264p-9f,
+                             -0x1.f03bdcp-11f, 0x1.1defc4p-11f, -0x1.0e2acep-12f};
+#pragma unroll
+    for (int v = 0; v < kV; ++v) P[v] = LN::all(kP[8]);
+#pragma unroll
+    for (int i = 7; i >= 0; --i)
+#pragma unroll
+      for (int v = 0; v < kV; ++v) P[v] = vfma(P[v], g[v], LN::all(kP[i]));
+#pragma unroll
+    for (int v = 0; v < kV; ++v) {
+      V nl = vfma(vmul(g[v], g[v]), P[v], g[v]);
+      nl = vfma(e[v], LN::all(0x1.62e430p-23f), nl);           // 2 ln u
+      float x[kL], y[kL];
+      LN::to(nl, x);
+#pragma unroll
+      for (int l = 0; l < kL; ++l)
+        asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y[l]) : "f"(fmaxf(-x[l], 1e-30f)));
+      const V ns = vmul(nl, LN::from(y));
+      nr[v] = vfma(vfma(ns, ns, nl), vmul(LN::from(y), LN::all(0.5f)), ns);
+    }
+  }
+  uint32_t qd[kN];                                             // (k + 2^21) 2^8
+  V t[kV], w[kV], sn[kV], cs[kV];
+#pragma unroll
+  for (int v = 0; v < kV; ++v) {
+    float j[kL];
+#pragma unroll
+    for (int l = 0; l < kL; ++l) {
+      qd[v * kL + l] = xb[v * kL + l] + 0x20000100u;
+      j[l] = __uint_as_float(((qd[v * kL + l] >> 8) & 0x3fffffu) | 0x4b000000u);   // 2^23 + j
+    }
+    t[v] = vfma(LN::from(j), LN::all(0x1p-21f), LN::all(-5.0f));
+    w[v] = vmul(t[v], t[v]);
+  }
+  constexpr float kS[4] = {-0x1.a0f38ap-26f, -0x1.4abbbap-4f, 0x1.465ee8p-9f, -0x1.2da132p-15f};
+  constexpr float kC[4] = {-0x1.3bd3ccp-2f, 0x1.03c1e2p-6f, -0x1.55c752p-12f, 0x1.da30fap-19f};
+#pragma unroll
+  for (int v = 0; v < kV; ++v) { sn[v] = LN::all(kS[3]); cs[v] = LN::all(kC[3]); }
+#pragma unroll
+  for (int i = 2; i >= 0; --i)
+#pragma unroll
+    for (int v = 0; v < kV; ++v) {
+      sn[v] = vfma(w[v], sn[v], LN::all(kS[i]));
+      cs[v] = vfma(w[v], cs[v], LN::all(kC[i]));
+    }
+#pragma unroll
+  for (int v = 0; v < kV; ++v) {
+    sn[v] = vfma(t[v], LN::all(0x1.921fb6p-1f), vmul(t[v], sn[v]));
+    cs[v] = vfma(w[v], cs[v], LN::all(1.0f));
+    float a[kL], b[kL], c[kL], s[kL];
+    LN::to(cs[v], a);
+    LN::to(sn[v], b);
+#pragma unroll
+    for (int l = 0; l < kL; ++l) {
+      const uint32_t q = qd[v * kL + l];
+      const bool odd = (q & 0x40000000u) != 0;
+      // cos is negative in quadrants 1 and 2, sin in 2 and 3; both negated, as nr is -rad
+      c[l] = __uint_as_float(__float_as_uint(odd ? b[l] : a[l]) ^ ((q + 0xc0000000u) & 0x80000000u));
+      s[l] = __uint_as_float(__float_as_uint(odd ? a[l] : b[l]) ^ (~q & 0x80000000u));
+    }
+    zc[v] = LN::from(c);
+    zs[v] = LN::from(s);
+  }
 }
 
-// Box-Muller on one pair of uniforms: (rad cos(2 pi ub), rad sin(2 pi ub)).
+// One pair of words.
 __device__ __forceinline__ float2 box_muller(uint32_t xa, uint32_t xb) {
-  const float ua = u01(xa);
-  const float ub = u01(xb);
-  const float rad = sqrtf(-2.0f * logf(ua));
-  float s, c;
-  sincospif(2.0f * ub, &s, &c);
-  return make_float2(rad * c, rad * s);
+  const uint32_t a[1] = {xa}, b[1] = {xb};
+  float nr[1], c[1], s[1];
+  box_muller_parts<1, float>(a, b, nr, c, s);
+  return make_float2(__fmul_rn(nr[0], c[0]), __fmul_rn(nr[0], s[0]));
+}
+// The four words of a counter, in packed arithmetic.
+__device__ __forceinline__ float4 box_muller4(uint4 x) {
+  const uint32_t a[2] = {x.x, x.z}, b[2] = {x.y, x.w};
+  float2 nr[1], c[1], s[1];
+  box_muller_parts<1, float2>(a, b, nr, c, s);
+  c[0] = mul2(nr[0], c[0]);
+  s[0] = mul2(nr[0], s[0]);
+  return make_float4(c[0].x, s[0].x, c[0].y, s[0].y);
 }
 
 // Four normals of counter word `c4` of the stream (seed, x1, x2, x3).
@@ -83,9 +225,7 @@ __device__ __forceinline__ float4 normal4(uint64_t seed, uint32_t c4, uint32_t x
                                           uint32_t x3) {
   const uint4 w = philox4x32_10(make_uint4(c4, x1, x2, x3), static_cast<uint32_t>(seed),
                                 static_cast<uint32_t>(seed >> 32));
-  const float2 a = box_muller(w.x, w.y);
-  const float2 b = box_muller(w.z, w.w);
-  return make_float4(a.x, a.y, b.x, b.y);
+  return box_muller4(w);
 }
 
 // ---------------------------------------------------------------------------
