@@ -768,7 +768,7 @@ def linear_measure(dev, wl, T, K, W, compare=True, e2e=True):
     out["launches"] = zb.zo_kernel_launches(z.ctx) - launches0
     z.sync()
     names = {1: "128x256", 2: "256x256", 3: "256x224", 4: "256x256 pair", 5: "256x240 pair",
-             6: "256x224 pair", 7: "256x192 pair", 8: "256x128 pair"}
+             6: "256x224 pair", 7: "256x192 pair", 8: "256x128 pair", 9: "few tokens"}
     out["tiling"] = []
     for i, (m, n) in enumerate(wl.shapes):
         zb.zo_linear_perturbed(z.ctx, i, X[n], Y[i])

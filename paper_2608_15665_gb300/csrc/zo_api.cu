@@ -48,6 +48,12 @@ void zo::set_last_error(const char* msg) { g_last_error = msg; }
 
 namespace {
 
+// Words of the linear route's flags and counters for a capacity of s_cap tokens: those of the
+// SM-pair launches' row blocks, then kLinearFewFlags of the few-token launches.
+int64_t s_flag_words(int64_t s_cap) {
+  return (s_cap / 256 + 1) * zo::kLinearPairCounters + zo::kLinearFewFlags;
+}
+
 // Makes a context's device current for the length of a call and gives the caller's back:
 // every kernel of a context runs on the device it was created on, whatever device the
 // calling thread has selected since.
@@ -165,6 +171,8 @@ struct zo_ctx {
 };
 
 namespace {
+
+int64_t s_flag_words(const zo_ctx* c) { return s_flag_words(c->s_cap); }
 
 void free_ctx(zo_ctx* c) {
   if (!c) return;
@@ -1054,6 +1062,68 @@ zo_status zo_linear_prepare(zo_ctx* c, uint32_t t, int32_t qa, float ca, int32_t
   return ZO_OK;
 }
 
+}  // extern "C"
+
+namespace {
+
+// The perturbed-linear route's workspace for T tokens and `part` floats of partial sums;
+// growing it synchronises the stream.
+zo_status linear_workspace(zo_ctx* c, int64_t T, int64_t part) {
+  const int64_t HLW = zo::tc_hl_width(c->r);
+  if (T > c->s_cap || part > c->part_cap) {
+    ZO_CUDA(cudaStreamSynchronize(c->stream), "stream synchronize");
+    if (T > c->s_cap) {
+      cudaFree(c->d_s_hl);
+      cudaFree(c->d_s_count);
+      cudaFree(c->d_s_flags);
+      c->d_s_hl = nullptr;
+      c->d_s_count = nullptr;
+      c->d_s_flags = nullptr;
+      c->s_cap = 0;
+      const int64_t cap = (T + 127) / 128 * 128;
+      const int64_t n_flags = s_flag_words(cap);
+      ZO_CUDA(cudaMalloc(&c->d_s_hl, sizeof(__nv_bfloat16) * cap * HLW), "cudaMalloc(S_HL)");
+      ZO_CUDA(cudaMalloc(&c->d_s_count, sizeof(uint32_t) * (cap / 32)), "cudaMalloc(S counters)");
+      ZO_CUDA(cudaMalloc(&c->d_s_flags, sizeof(uint32_t) * n_flags),
+              "cudaMalloc(S row-block counters)");
+      // on the context's stream: a plain cudaMemset runs on the legacy default stream,
+      // which a non-blocking stream's kernels are not ordered after
+      ZO_CUDA(cudaMemsetAsync(c->d_s_count, 0, sizeof(uint32_t) * (cap / 32), c->stream),
+              "zero S counters");
+      ZO_CUDA(cudaMemsetAsync(c->d_s_flags, 0, sizeof(uint32_t) * n_flags, c->stream),
+              "zero S row-block counters");
+      c->lin_epoch = 0;
+      c->s_cap = cap;
+    }
+    if (part > c->part_cap) {
+      cudaFree(c->d_s_part);
+      c->d_s_part = nullptr;
+      c->part_cap = 0;
+      ZO_CUDA(cudaMalloc(&c->d_s_part, sizeof(float) * part), "cudaMalloc(partial S)");
+      c->part_cap = part;
+    }
+  }
+  return ZO_OK;
+}
+
+// The epoch of the next launch that counts in the row-block flags and counters.
+zo_status linear_epoch(zo_ctx* c, uint32_t* epoch) {
+  if (c->lin_epoch + 1 >= zo::kLinearPairEpochs) {
+    // the epochs start again: no flag or counter may hold an old call's
+    ZO_CUDA(cudaMemsetAsync(c->d_s_flags, 0,
+                            sizeof(uint32_t) * s_flag_words(c),
+                            c->stream),
+            "zero S row-block counters");
+    c->lin_epoch = 0;
+  }
+  *epoch = ++c->lin_epoch;
+  return ZO_OK;
+}
+
+}  // namespace
+
+extern "C" {
+
 zo_status zo_linear_perturbed(zo_ctx* c, int32_t mat, const void* X, int64_t T, int64_t ldx,
                               void* Y, int64_t ldy) {
   if (!c || !X || !Y) return ZO_ERR_INVALID_ARG;
@@ -1079,6 +1149,39 @@ zo_status zo_linear_perturbed(zo_ctx* c, int32_t mat, const void* X, int64_t T, 
   }
   const int32_t r = c->r;
   const int64_t HLW = zo::tc_hl_width(r);
+  // few tokens, automatic tiling: every SM a few columns of Y
+  const zo::LinearFewPlan few = c->linear_tile == 0 ? zo::linear_few_plan(T, m, n, r, c->sms)
+                                                    : zo::LinearFewPlan{};
+  if (few.ctas > 0) {
+    const zo_status ws = linear_workspace(c, T, T * r);
+    if (ws != ZO_OK) return ws;
+    CUtensorMap tm_x{}, tm_xs{}, tm_w{}, tm_pk{}, tm_s{}, tm_u{};
+    void* x = const_cast<void*>(X);
+    if (!encode_bf16_2d(&tm_x, x, n, T, ldx * 2, 64, (uint32_t)few.tokens) ||
+        !encode_bf16_2d(&tm_xs, x, n, T, ldx * 2, 64, (uint32_t)few.s_tokens) ||
+        !encode_bf16_2d(&tm_w, md.W, n, m, md.ldw * 2, 64, (uint32_t)few.cols) ||
+        !encode_bf16_2d(&tm_pk, c->d_pk + c->h_pk_off[mat], n, 2 * r, (n + 63) / 64 * 64 * 2, 64,
+                        (uint32_t)few.s_cols) ||
+        !encode_bf16_2d(&tm_s, c->d_s_hl, HLW, T, HLW * 2, 64, (uint32_t)few.tokens) ||
+        !encode_bf16_2d(&tm_u, c->d_u_lin, HLW, c->u_rows, HLW * 2, 64, (uint32_t)few.cols)) {
+      g_last_error = "zo_linear_perturbed: cuTensorMapEncodeTiled rejected a descriptor";
+      return ZO_ERR_CUDA;
+    }
+    uint32_t epoch = 0;
+    const zo_status es = linear_epoch(c, &epoch);
+    if (es != ZO_OK) return es;
+    const bool inject = c->inject_wait;    // the test hook is one-shot
+    c->inject_wait = false;
+    ZO_CUDA(zo::launch_linear_few(tm_x, tm_xs, tm_w, tm_pk, tm_s, tm_u, few, T, m, n, r,
+                                  c->h_tc[mat].u_row0, c->d_s_hl,
+                                  c->d_s_flags + s_flag_words(c) - zo::kLinearFewFlags, epoch,
+                                  static_cast<__nv_bfloat16*>(Y), ldy, inject, c->d_status,
+                                  c->stream),
+            "perturbed linear kernel (few tokens)");
+    c->launches += 1;
+    c->last_linear_tiling = zo::kLinearFewTiling;
+    return ZO_OK;
+  }
   // the Y GEMM's tiling: automatic = the pair tiling whose busiest pair has the least
   // operand traffic (the single-CTA tilings if no cluster of the pair kernel fits), or the
   // one ZO_OPTION_LINEAR_TILE names
@@ -1112,39 +1215,8 @@ zo_status zo_linear_perturbed(zo_ctx* c, int32_t mat, const void* X, int64_t T, 
     zo::linear_s_split(T, n, c->sms, &k_split, &k_chunk);
   }
   const int64_t part = (int64_t)k_split * T * r;
-  if (T > c->s_cap || part > c->part_cap) {
-    ZO_CUDA(cudaStreamSynchronize(c->stream), "stream synchronize");
-    if (T > c->s_cap) {
-      cudaFree(c->d_s_hl);
-      cudaFree(c->d_s_count);
-      cudaFree(c->d_s_flags);
-      c->d_s_hl = nullptr;
-      c->d_s_count = nullptr;
-      c->d_s_flags = nullptr;
-      c->s_cap = 0;
-      const int64_t cap = (T + 127) / 128 * 128;
-      const int64_t n_flags = (cap / 256 + 1) * zo::kLinearPairCounters;
-      ZO_CUDA(cudaMalloc(&c->d_s_hl, sizeof(__nv_bfloat16) * cap * HLW), "cudaMalloc(S_HL)");
-      ZO_CUDA(cudaMalloc(&c->d_s_count, sizeof(uint32_t) * (cap / 32)), "cudaMalloc(S counters)");
-      ZO_CUDA(cudaMalloc(&c->d_s_flags, sizeof(uint32_t) * n_flags),
-              "cudaMalloc(S row-block counters)");
-      // on the context's stream: a plain cudaMemset runs on the legacy default stream,
-      // which a non-blocking stream's kernels are not ordered after
-      ZO_CUDA(cudaMemsetAsync(c->d_s_count, 0, sizeof(uint32_t) * (cap / 32), c->stream),
-              "zero S counters");
-      ZO_CUDA(cudaMemsetAsync(c->d_s_flags, 0, sizeof(uint32_t) * n_flags, c->stream),
-              "zero S row-block counters");
-      c->lin_epoch = 0;
-      c->s_cap = cap;
-    }
-    if (part > c->part_cap) {
-      cudaFree(c->d_s_part);
-      c->d_s_part = nullptr;
-      c->part_cap = 0;
-      ZO_CUDA(cudaMalloc(&c->d_s_part, sizeof(float) * part), "cudaMalloc(partial S)");
-      c->part_cap = part;
-    }
-  }
+  const zo_status st = linear_workspace(c, T, part);
+  if (st != ZO_OK) return st;
   const bool narrow_y = pair_n == 0 && zo::linear_y_tile_cols(tiling) % 64 != 0;
   CUtensorMap tm_x{}, tm_pk{}, tm_s{}, tm_y{}, tm_w{}, tm_u{}, tm_pk_half{}, tm_ps{};
   bool enc =
@@ -1175,20 +1247,14 @@ zo_status zo_linear_perturbed(zo_ctx* c, int32_t mat, const void* X, int64_t T, 
   }
   if (pair_n > 0) {
     // one launch: S = X P^T (in contributor tiles or S tiles) and Y = X W^T + S U^T
-    if (c->lin_epoch + 1 >= zo::kLinearPairEpochs) {
-      // the epochs start again: no counter may hold an old call's complete count
-      ZO_CUDA(cudaMemsetAsync(c->d_s_flags, 0,
-                              sizeof(uint32_t) * (c->s_cap / 256 + 1) * zo::kLinearPairCounters,
-                              c->stream),
-              "zero S row-block counters");
-      c->lin_epoch = 0;
-    }
-    ++c->lin_epoch;
+    uint32_t epoch = 0;
+    const zo_status es = linear_epoch(c, &epoch);
+    if (es != ZO_OK) return es;
     const bool inject = c->inject_wait;    // the test hook is one-shot
     c->inject_wait = false;
     ZO_CUDA(zo::launch_linear_pair(tm_x, tm_w, tm_s, tm_u, tm_y, tm_pk_half, tm_ps, T, m, n,
                                    c->h_tc[mat].u_row0, r, tiling, plan, c->d_s_hl, c->d_s_part,
-                                   c->d_s_flags, c->lin_epoch, inject, c->d_status, c->stream),
+                                   c->d_s_flags, epoch, inject, c->d_status, c->stream),
             "perturbed linear kernel (SM pairs)");
     c->launches += 1;
   } else {
@@ -1243,7 +1309,7 @@ zo_status zo_sync_status(zo_ctx* c) {
               "zero S counters");
     if ((s & zo::kDevTimeout) && c->d_s_flags) {
       ZO_CUDA(cudaMemsetAsync(c->d_s_flags, 0,
-                              sizeof(uint32_t) * (c->s_cap / 256 + 1) * zo::kLinearPairCounters,
+                              sizeof(uint32_t) * s_flag_words(c),
                               c->stream),
               "zero S row-block counters");
       c->lin_epoch = 0;

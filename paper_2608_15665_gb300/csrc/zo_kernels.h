@@ -248,6 +248,30 @@ constexpr uint32_t kLinearPairCountsPerCall = 8;   // 32-row groups of a 256-row
 constexpr int32_t kLinearPairCounters = 40;        // flags and counters per 256-row block
 constexpr uint32_t kLinearPairEpochs = 1u << 26;
 
+// The layer for at most 128 tokens (zo_linear_few.cu): CTAs of all the tokens x `cols` columns
+// of Y, after n_s CTAs of S (s_tokens x s_cols each), one wave on the device's SMs; ctas = 0:
+// not for this shape.  Reported as tiling kLinearFewTiling.
+constexpr int32_t kLinearFewTiling = 9;
+constexpr int32_t kLinearFewFlags = 32;      // words of flags
+struct LinearFewPlan {
+  int32_t tokens, cols, n_s, s_tokens, s_cols, ctas, panels, s_panels, stages, s_stages;
+  int64_t smem;
+};
+LinearFewPlan linear_few_plan(int64_t T, int64_t m, int64_t n, int32_t r, int32_t sms);
+// tm_x over X (box 64 x plan.tokens), tm_xs over X (box 64 x plan.s_tokens), tm_w over W_i
+// (box 64 x plan.cols), tm_pk over P_K (box 64 x plan.s_cols), tm_s over s_hl (box 64 x
+// plan.tokens), tm_u over the bf16 U operand (box 64 x plan.cols; W_i's rows from u_row0).
+// flags: kLinearFewFlags words, none of which holds epoch before the launch.  inject_wait
+// (test hook): the CTAs wait for S, with the short test limit, for an epoch that never comes;
+// the launch then reports kDevTimeout.
+cudaError_t launch_linear_few(const CUtensorMap& tm_x, const CUtensorMap& tm_xs,
+                              const CUtensorMap& tm_w, const CUtensorMap& tm_pk,
+                              const CUtensorMap& tm_s, const CUtensorMap& tm_u,
+                              const LinearFewPlan& plan, int64_t T, int64_t m, int64_t n, int32_t r,
+                              int32_t u_row0, __nv_bfloat16* s_hl, uint32_t* flags, uint32_t epoch,
+                              __nv_bfloat16* Y, int64_t ldy, bool inject_wait, uint32_t* d_status,
+                              cudaStream_t s);
+
 // ---- refresh of tall panels at r = 16 ... 128: CholeskyQR2 (zo_cholqr.cu) ----------
 constexpr int32_t kCqChunkRows = 1024;   // rows per partial Gram matrix
 struct CqPanel {

@@ -138,56 +138,10 @@ __device__ __forceinline__ uint32_t count_epoch(uint32_t* f, uint32_t epoch) {
     cur = prev;
   }
 }
-__device__ __forceinline__ void set_ready(uint32_t* f, uint32_t epoch) {
-  asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(f), "r"(epoch) : "memory");
-}
-// every one of the n (<= 32) flags at f holds epoch (bounded; false on abort or timeout).
-// Each poll issues the n loads together (relaxed, independent, so they overlap in one L2
-// round trip -- acquire loads would complete one after another); once all match, one
-// acquire-release fence gives the acquire.
-__device__ __forceinline__ bool wait_s_rows(const uint32_t* f, int n, uint32_t epoch,
-                                            const volatile int* abort, long long limit_cycles) {
-  const long long t0 = clock64();
-  for (;;) {
-    uint32_t v[32];
-#pragma unroll
-    for (int j = 0; j < 32; ++j) {
-      v[j] = epoch;
-      if (j < n)
-        asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v[j]) : "l"(f + j) : "memory");
-    }
-    bool all = true;
-#pragma unroll
-    for (int j = 0; j < 32; ++j) all = all && v[j] == epoch;
-    if (all) {
-      asm volatile("fence.acq_rel.gpu;" ::: "memory");
-      return true;
-    }
-    if (*abort) return false;
-    if (clock64() - t0 > limit_cycles) return false;
-    __nanosleep(64);
-  }
-}
-// generic-proxy global writes <-> later async-proxy (TMA) reads
-__device__ __forceinline__ void fence_async_global() {
-  asm volatile("fence.proxy.async.global;" ::: "memory");
-}
-
 __device__ __forceinline__ void lp_give_up(LinPairShared& sh, uint32_t* status) {
   atomicOr(status, (uint32_t)kDevTimeout);
   *reinterpret_cast<volatile int*>(&sh.abort_flag) = 1;
   store_peer(&sh.abort_flag, 1);
-}
-
-// 32 lanes x 16 consecutive 32-bit columns: thread t gets lane (base lane + t)
-__device__ __forceinline__ void tmem_ld_32x32b_x16(uint32_t taddr, uint32_t (&v)[16]) {
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
-      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
-      : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]),
-        "=r"(v[7]), "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]),
-        "=r"(v[14]), "=r"(v[15])
-      : "r"(taddr));
 }
 
 // Columns kC j .. kC j + kC - 1 of S for this thread's row (kC = min(R, 32)): the sum of
