@@ -104,6 +104,11 @@ struct zo_ctx {
   float* d_cq_partial = nullptr;
   float* d_cq_linv = nullptr;
   int32_t n_cq_panels = 0, n_cq_chunks = 0;
+  // panels at r = 4 and 8 held in registers: short ones first, then the tall ones by the CTAs
+  // that hold one (1, 2, 4, 8)
+  zo::CqPanel* d_small = nullptr;
+  int32_t n_short = 0;
+  int32_t n_small[4] = {0, 0, 0, 0};
   std::vector<int64_t> up_off, up_cnt, down_off, down_cnt;   // per level, into d_qr_blocks
   uint32_t* d_status = nullptr;
   int path_option = 0;
@@ -187,6 +192,7 @@ void free_ctx(zo_ctx* c) {
   cudaFree(c->d_qr_ws);
   cudaFree(c->d_qr_blocks);
   cudaFree(c->d_cq_panels);
+  cudaFree(c->d_small);
   cudaFree(c->d_cq_chunks);
   cudaFree(c->d_cq_partial);
   cudaFree(c->d_cq_linv);
@@ -697,11 +703,15 @@ zo_status zo_create(zo_ctx** out, const zo_matrix* mats, int32_t n_mats, int32_t
   int64_t qr_floats = 0;
   // a panel with rows >= 4r has kappa(Omega) <= ~3, well inside CholeskyQR2's range
   auto use_cholqr = [&](int64_t rows) { return zo::cholqr_supported(r) && rows >= 4 * (int64_t)r; };
+  auto use_small = [&](int64_t rows) {
+    return zo::cholqr_small_short(r, rows) || zo::cholqr_small_ctas(r, rows) > 0;
+  };
+  auto use_tsqr = [&](int64_t rows) { return !use_cholqr(rows) && !use_small(rows); };
   {
     std::vector<QrLevel> dry;
     for (int32_t i = 0; i < n_mats; ++i) {
-      if (!use_cholqr(mats[i].m)) plan_panel(nullptr, mats[i].m, r, 0, zo::kTagOmegaU, B, dry, nullptr, &qr_floats);
-      if (!use_cholqr(mats[i].n)) plan_panel(nullptr, mats[i].n, r, 0, zo::kTagOmegaV, B, dry, nullptr, &qr_floats);
+      if (use_tsqr(mats[i].m)) plan_panel(nullptr, mats[i].m, r, 0, zo::kTagOmegaU, B, dry, nullptr, &qr_floats);
+      if (use_tsqr(mats[i].n)) plan_panel(nullptr, mats[i].n, r, 0, zo::kTagOmegaV, B, dry, nullptr, &qr_floats);
     }
   }
   e = cudaMalloc(&c->d_qr_ws, sizeof(float) * std::max<int64_t>(qr_floats, 4));
@@ -722,13 +732,27 @@ zo_status zo_create(zo_ctx** out, const zo_matrix* mats, int32_t n_mats, int32_t
     }
     cq_panels.push_back(p);
   };
+  std::vector<zo::CqPanel> small[5];     // short ones, then tall ones of 1, 2, 4, 8 CTAs
+  auto add_panel = [&](float* out, int64_t rows, uint32_t gidx, uint32_t tag) {
+    if (use_cholqr(rows)) {
+      add_cholqr(out, rows, gidx, tag);
+    } else if (use_small(rows)) {
+      const int32_t ctas = zo::cholqr_small_ctas(r, rows);
+      small[ctas == 0 ? 0 : ctas == 1 ? 1 : ctas == 2 ? 2 : ctas == 4 ? 3 : 4].push_back(
+          {out, rows, gidx, tag, 0, 0});
+    } else {
+      plan_panel(out, rows, r, gidx, tag, B, levels, c->d_qr_ws, &off);
+    }
+  };
   for (int32_t i = 0; i < n_mats; ++i) {
     const uint32_t gidx = matrix_index_base + (uint32_t)i;
-    if (use_cholqr(mats[i].m)) add_cholqr(mats[i].U, mats[i].m, gidx, zo::kTagOmegaU);
-    else plan_panel(mats[i].U, mats[i].m, r, gidx, zo::kTagOmegaU, B, levels, c->d_qr_ws, &off);
-    if (use_cholqr(mats[i].n)) add_cholqr(mats[i].V, mats[i].n, gidx, zo::kTagOmegaV);
-    else plan_panel(mats[i].V, mats[i].n, r, gidx, zo::kTagOmegaV, B, levels, c->d_qr_ws, &off);
+    add_panel(mats[i].U, mats[i].m, gidx, zo::kTagOmegaU);
+    add_panel(mats[i].V, mats[i].n, gidx, zo::kTagOmegaV);
   }
+  std::vector<zo::CqPanel> small_panels;
+  for (const auto& v : small) small_panels.insert(small_panels.end(), v.begin(), v.end());
+  c->n_short = (int32_t)small[0].size();
+  for (int k = 0; k < 4; ++k) c->n_small[k] = (int32_t)small[k + 1].size();
   c->n_cq_panels = (int32_t)cq_panels.size();
   c->n_cq_chunks = (int32_t)cq_chunks.size();
   std::vector<zo::QrBlock> all_blocks;
@@ -749,6 +773,8 @@ zo_status zo_create(zo_ctx** out, const zo_matrix* mats, int32_t n_mats, int32_t
   if (e == cudaSuccess) e = cudaMalloc(&c->d_proj_units, sizeof(int2) * std::max<size_t>(units.size(), 1));
   if (e == cudaSuccess) e = cudaMalloc(&c->d_qr_blocks, sizeof(zo::QrBlock) * std::max<size_t>(all_blocks.size(), 1));
   if (e == cudaSuccess) e = cudaMalloc(&c->d_status, sizeof(uint32_t));
+  if (e == cudaSuccess && !small_panels.empty())
+    e = cudaMalloc(&c->d_small, sizeof(zo::CqPanel) * small_panels.size());
   if (e == cudaSuccess && c->n_cq_panels > 0) {
     e = cudaMalloc(&c->d_cq_panels, sizeof(zo::CqPanel) * cq_panels.size());
     if (e == cudaSuccess) e = cudaMalloc(&c->d_cq_chunks, sizeof(zo::CqChunk) * cq_chunks.size());
@@ -770,6 +796,9 @@ zo_status zo_create(zo_ctx** out, const zo_matrix* mats, int32_t n_mats, int32_t
     e = cudaMemcpy(c->d_proj_units, units.data(), sizeof(int2) * units.size(), cudaMemcpyHostToDevice);
   if (e == cudaSuccess && !all_blocks.empty())
     e = cudaMemcpy(c->d_qr_blocks, all_blocks.data(), sizeof(zo::QrBlock) * all_blocks.size(),
+                   cudaMemcpyHostToDevice);
+  if (e == cudaSuccess && !small_panels.empty())
+    e = cudaMemcpy(c->d_small, small_panels.data(), sizeof(zo::CqPanel) * small_panels.size(),
                    cudaMemcpyHostToDevice);
   if (e == cudaSuccess && c->n_cq_panels > 0)
     e = cudaMemcpy(c->d_cq_panels, cq_panels.data(), sizeof(zo::CqPanel) * cq_panels.size(),
@@ -823,6 +852,17 @@ zo_status zo_refresh(zo_ctx* c, uint32_t refresh_idx, int32_t reset_moments) {
                                c->d_status, c->stream),
             "refresh down-pass kernel");
     ++c->launches;
+  }
+  const zo::CqPanel* tall = c->d_small + c->n_short;
+  for (int k = 0; k < 4; ++k) {
+    const int32_t n_short = k == 0 ? c->n_short : 0;
+    if (c->n_small[k] > 0 || n_short > 0) {
+      ZO_CUDA(zo::launch_cholqr_small(tall, c->n_small[k], c->d_small, n_short, 1 << k, c->r,
+                                      c->seed, refresh_idx, c->d_status, c->stream),
+              "refresh kernel (panels in registers)");
+      ++c->launches;
+    }
+    tall += c->n_small[k];
   }
   if (c->n_cq_panels > 0) {
     ZO_CUDA(zo::launch_cholqr(c->d_cq_panels, c->n_cq_panels, c->d_cq_chunks, c->n_cq_chunks,

@@ -294,6 +294,16 @@ cudaError_t launch_cholqr(const CqPanel* d_panels, int32_t n_panels, const CqChu
                           int32_t n_chunks, float* d_partial, float* d_linv, int32_t r,
                           uint64_t seed, uint32_t refresh_idx, uint32_t* d_status, cudaStream_t s);
 
+// ---- refresh at r = 4 and 8 with the panel in registers (zo_cholqr_small.cu) -----------
+// CTAs (a cluster of 1, 2, 4 or 8) that hold a tall panel, 0 if it is not for this kernel;
+// and whether a panel is one of its short ones (fewer than 4 r rows).
+int32_t cholqr_small_ctas(int32_t r, int64_t rows);
+bool cholqr_small_short(int32_t r, int64_t rows);
+// One launch: n_tall tall panels of the same `ctas`, and (ctas = 1) n_short short ones.
+cudaError_t launch_cholqr_small(const CqPanel* d_tall, int32_t n_tall, const CqPanel* d_short,
+                                int32_t n_short, int32_t ctas, int32_t r, uint64_t seed,
+                                uint32_t refresh_idx, uint32_t* d_status, cudaStream_t s);
+
 // ---- refresh: batched TSQR + sign correction (zo_qr.cu) ------------------------
 int32_t qr_block_rows(int32_t r);
 cudaError_t launch_qr_up(const QrBlock* d_blocks, int32_t n_blocks, int32_t r, uint64_t seed,

@@ -24,6 +24,7 @@
 // Blocks with fewer real rows than B are padded with zero rows, which leaves the
 // factorisation of the real rows unchanged and produces zero rows of Q there.
 #include "zo_kernels.h"
+#include "zo_reduce.cuh"
 
 namespace zo {
 namespace {
@@ -48,32 +49,6 @@ struct QrSmem {
   float diag[R];               // beta_j = R_jj
   float tau[R];
 };
-
-// Recursive-halving reduction of R per-lane values across a warp.  Afterwards
-// lane l holds the warp sum of element c = l * (R/32) + k (k < R/32) when R >= 32,
-// or of element c = l / (32/R) (in p[0]) when R < 32.
-template <int R>
-__device__ __forceinline__ void warp_reduce_scatter(float (&p)[R], int lane) {
-#pragma unroll
-  for (int s = 0; s < 5; ++s) {
-    const int o = 16 >> s;
-    const int size = R >> s;
-    if (size >= 2) {
-      const int half = size >> 1;
-      const bool upper = (lane & o) != 0;
-#pragma unroll
-      for (int i = 0; i < R / 2; ++i) {
-        if (i < half) {
-          const float send = upper ? p[i] : p[i + half];
-          const float keep = upper ? p[i + half] : p[i];
-          p[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
-        }
-      }
-    } else {
-      p[0] += __shfl_xor_sync(0xffffffffu, p[0], o);
-    }
-  }
-}
 
 // Block-wide sum of H per-thread values (columns off .. off+H-1) into
 // red[warp][off + c] (one partial per warp).
