@@ -11,8 +11,17 @@
 //            SGD:  D = G                                              (Sec. 3)
 //            C_i = -lr D + restore_coef eps Z_i^(restore_query)
 // P_i = C_i V_i^T (r x n) then feeds the weight pass.  For the tensor-core path the kernel
-// also writes max |C_i| (p.amax), from which the pass's operand scale is chosen.
+// also writes C_i as the projection's operand, rows [hi | lo] of the fp16 pair of
+// C_i 2^(e_C,i) with e_C,i from max |C_i| (zo_tc_common.cuh), and pinv_i = 2^-(e_P,i).
+//
+// One CTA per matrix up to r = 32, a cluster of four at r = 64 and of eight at r = 128 (the
+// maximum and the norm meet through distributed shared memory): at most two counters per
+// thread.  Latency-bound: the perturbation's draws, which need no memory, come before the
+// wait for the stream's previous kernel.
+#include "zo_cluster.cuh"
 #include "zo_kernels.h"
+#include "zo_launch.cuh"
+#include "zo_tc_common.cuh"
 
 namespace zo {
 namespace {
@@ -26,19 +35,43 @@ __device__ __forceinline__ float4 f4_scale(float a, float4 x) {
   return make_float4(a * x.x, a * x.y, a * x.z, a * x.w);
 }
 
-__global__ void __launch_bounds__(256) coeff_kernel(const MatDesc* __restrict__ mats,
-                                                    CoeffParams p) {
-  __shared__ float rho_s[kMaxQ];
-  __shared__ float red_s[8];
-  __shared__ float max_s[8];
-  const MatDesc md = mats[blockIdx.x];
-  const int r = p.r;
-  const int rr = r * r;          // r is a multiple of 4, so rr is a multiple of 16
-  const int n_ctr = rr / 4;
-  const int tid = threadIdx.x;
+constexpr int kCoeffThreads = 256;
+constexpr int kCoeffIters = 2;              // counters per thread
+__host__ __device__ constexpr int coeff_ctas(int r) { return r == 128 ? 8 : r == 64 ? 4 : 1; }
 
+__global__ void __launch_bounds__(kCoeffThreads)
+coeff_kernel(const MatDesc* __restrict__ mats, const CoeffParams p) {
+  extern __shared__ float rho_s[];          // q values (step mode)
+  __shared__ float sum_s[8], max_s[8];
+  __shared__ float cta_sum, cta_max;
+  const int r = p.r, ctas = coeff_ctas(r);
+  const int i = (int)(blockIdx.x / ctas), rank = (int)(blockIdx.x % ctas);
+  const MatDesc md = mats[i];
+  const int n_ctr = r * r / 4;              // r is a multiple of 4, so r * r of 16
+  const int per = n_ctr / ctas;             // this CTA's counters
+  const int c0 = rank * per;
+  const int tid = threadIdx.x;
+  float4 out[kCoeffIters];
+
+  if (p.mode == kCoeffPerturb) {
+#pragma unroll
+    for (int k = 0; k < kCoeffIters; ++k) {
+      const int c = tid + k * kCoeffThreads;
+      if (c >= per) break;
+      float4 acc = f4_scale(p.ca, normal4(p.seed, (uint32_t)(c0 + c), md.gidx, p.t,
+                                          query_word(kTagZ, (uint32_t)p.qa)));
+      if (p.qb >= 0)
+        acc = f4_axpy(p.cb, normal4(p.seed, (uint32_t)(c0 + c), md.gidx, p.t,
+                                    query_word(kTagZ, (uint32_t)p.qb)), acc);
+      out[k] = f4_scale(p.eps, acc);
+    }
+  }
+  pdl_wait();
+  pdl_trigger();
+
+  float gsq = 0.0f;
   if (p.mode == kCoeffStep) {
-    for (int k = tid; k < p.q; k += blockDim.x) {
+    for (int k = tid; k < p.q; k += kCoeffThreads) {
       float rho;
       if (p.scheme == 0) {          // central: (L+_k - L-_k) / (2 eps)
         rho = (p.losses[2 * k] - p.losses[2 * k + 1]) / (2.0f * p.eps);
@@ -50,21 +83,10 @@ __global__ void __launch_bounds__(256) coeff_kernel(const MatDesc* __restrict__ 
       rho_s[k] = rho;
     }
     __syncthreads();
-  }
-
-  float gsq = 0.0f;
-  float cmax = 0.0f;
-  float4* C4 = reinterpret_cast<float4*>(md.C);
-  for (int c = tid; c < n_ctr; c += blockDim.x) {
-    float4 out;
-    if (p.mode == kCoeffPerturb) {
-      float4 acc = f4_scale(p.ca, normal4(p.seed, (uint32_t)c, md.gidx, p.t,
-                                          query_word(kTagZ, (uint32_t)p.qa)));
-      if (p.qb >= 0)
-        acc = f4_axpy(p.cb, normal4(p.seed, (uint32_t)c, md.gidx, p.t,
-                                    query_word(kTagZ, (uint32_t)p.qb)), acc);
-      out = f4_scale(p.eps, acc);
-    } else {
+#pragma unroll
+    for (int it = 0; it < kCoeffIters; ++it) {
+      if (tid + it * kCoeffThreads >= per) break;
+      const int c = c0 + tid + it * kCoeffThreads;
       // G: accumulate in query order, then divide by q (Alg. 3)
       float4 g = make_float4(0.f, 0.f, 0.f, 0.f);
       for (int k = 0; k < p.q; ++k)
@@ -93,40 +115,78 @@ __global__ void __launch_bounds__(256) coeff_kernel(const MatDesc* __restrict__ 
       } else {
         d = g;
       }
-      out = f4_scale(-p.lr, d);
+      out[it] = f4_scale(-p.lr, d);
       if (p.restore_query >= 0) {
         const float4 z = normal4(p.seed, (uint32_t)c, md.gidx, p.t,
                                  query_word(kTagZ, (uint32_t)p.restore_query));
-        out = f4_axpy(p.restore_coef * p.eps, z, out);
+        out[it] = f4_axpy(p.restore_coef * p.eps, z, out[it]);
       }
     }
-    C4[c] = out;
-    cmax = fmaxf(cmax, fmaxf(fmaxf(fabsf(out.x), fabsf(out.y)), fmaxf(fabsf(out.z), fabsf(out.w))));
   }
 
-  if (p.amax != nullptr) {
+  float cmax = 0.0f;
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) cmax = fmaxf(cmax, __shfl_xor_sync(0xffffffffu, cmax, o));
-    if ((tid & 31) == 0) max_s[tid >> 5] = cmax;
-    __syncthreads();
-    if (tid == 0) {
-      float m = 0.f;
-      for (int w = 0; w < (int)(blockDim.x >> 5); ++w) m = fmaxf(m, max_s[w]);
-      p.amax[blockIdx.x] = m;
-    }
+  for (int it = 0; it < kCoeffIters; ++it) {
+    if (tid + it * kCoeffThreads >= per) break;
+    const float4 o = out[it];
+    reinterpret_cast<float4*>(md.C)[c0 + tid + it * kCoeffThreads] = o;
+    cmax = fmaxf(cmax, fmaxf(fmaxf(fabsf(o.x), fabsf(o.y)), fmaxf(fabsf(o.z), fabsf(o.w))));
   }
+  const bool gamma = p.mode == kCoeffStep && p.gamma_out != nullptr;
+  if (p.c_hl == nullptr && !gamma) return;
 
-  if (p.mode == kCoeffStep && p.gamma_out != nullptr) {
+  // max |C_i| and sum G_i^2 over the CTA, then (in rank order) the cluster
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) gsq += __shfl_xor_sync(0xffffffffu, gsq, o);
-    if ((tid & 31) == 0) red_s[tid >> 5] = gsq;
-    __syncthreads();
+  for (int o = 16; o > 0; o >>= 1) {
+    cmax = fmaxf(cmax, __shfl_xor_sync(0xffffffffu, cmax, o));
+    gsq += __shfl_xor_sync(0xffffffffu, gsq, o);
+  }
+  if ((tid & 31) == 0) {
+    max_s[tid >> 5] = cmax;
+    sum_s[tid >> 5] = gsq;
+  }
+  __syncthreads();
+  cmax = gsq = 0.f;
+#pragma unroll
+  for (int w = 0; w < kCoeffThreads / 32; ++w) {
+    cmax = fmaxf(cmax, max_s[w]);
+    gsq += sum_s[w];
+  }
+  if (ctas > 1) {
     if (tid == 0) {
-      float s = 0.f;
-      for (int w = 0; w < (int)(blockDim.x >> 5); ++w) s += red_s[w];
-      p.gamma_out[blockIdx.x] = sqrtf(s);
+      cta_max = cmax;
+      cta_sum = gsq;
+    }
+    cta2::cluster_sync_all();
+    cmax = gsq = 0.f;
+    for (int c = 0; c < ctas; ++c) {
+      float m, g;
+      asm volatile("ld.shared::cluster.f32 %0, [%1];"
+                   : "=f"(m) : "r"(cta2::map_to(&cta_max, (uint32_t)c)) : "memory");
+      asm volatile("ld.shared::cluster.f32 %0, [%1];"
+                   : "=f"(g) : "r"(cta2::map_to(&cta_sum, (uint32_t)c)) : "memory");
+      cmax = fmaxf(cmax, m);
+      gsq += g;
     }
   }
+  if (gamma && rank == 0 && tid == 0) p.gamma_out[i] = sqrtf(gsq);
+  if (p.c_hl != nullptr) {
+    const int e_c = tc::coeff_scale_exp(cmax);
+    if (rank == 0 && tid == 0) p.pinv[i] = tc::exp2i(-(e_c + tc::p_scale_offset(r)));
+    const float scale = tc::exp2i(e_c);
+    const int width = tc::hl_width(r);
+#pragma unroll
+    for (int it = 0; it < kCoeffIters; ++it) {
+      if (tid + it * kCoeffThreads >= per) break;
+      const int e = 4 * (c0 + tid + it * kCoeffThreads);
+      uint2 hi, lo;
+      tc::split4_f16(out[it], scale, hi, lo);
+      uint16_t* row = p.c_hl + ((int64_t)i * r + e / r) * width + e % r;
+      *reinterpret_cast<uint2*>(row) = hi;
+      *reinterpret_cast<uint2*>(row + r) = lo;
+    }
+  }
+  if (ctas > 1) cta2::cluster_sync_all();   // the peers have read this CTA's values
 }
 
 // P[a][j] = sum_b C[a][b] V[j][b]; one thread per column j, rows a split over ty.
@@ -137,6 +197,8 @@ __global__ void __launch_bounds__(256) project_fma_kernel(const MatDesc* __restr
   const int2 u = units[blockIdx.x];
   const MatDesc md = mats[u.x];
   const int tid = threadIdx.x;
+  pdl_wait();
+  pdl_trigger();
   for (int e = tid; e < R * R; e += blockDim.x) Cs[e] = md.C[e];
   __syncthreads();
   const int64_t j = (int64_t)u.y + (tid & 127);
@@ -172,18 +234,20 @@ cudaError_t launch_project_fma_r(const MatDesc* d_mats, const int2* d_units, int
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
   }
-  project_fma_kernel<R><<<n_units, 256, smem, s>>>(d_mats, d_units);
-  return cudaGetLastError();
+  return launch_dependent(project_fma_kernel<R>, (unsigned)n_units, 256, smem, s, 1, true, d_mats,
+                          d_units);
 }
 
 }  // namespace
 
 cudaError_t launch_coeff(const MatDesc* d_mats, int32_t n_mats, const CoeffParams& p,
-                         cudaStream_t s) {
+                         bool dependent, cudaStream_t s) {
   if (n_mats <= 0) return cudaSuccess;
   if (p.q > kMaxQ) return cudaErrorInvalidValue;
-  coeff_kernel<<<n_mats, 256, 0, s>>>(d_mats, p);
-  return cudaGetLastError();
+  const unsigned ctas = (unsigned)coeff_ctas(p.r);
+  const size_t smem = p.mode == kCoeffStep ? sizeof(float) * p.q : 0;
+  return launch_dependent(coeff_kernel, (unsigned)n_mats * ctas, kCoeffThreads, smem, s, ctas,
+                          dependent, d_mats, p);
 }
 
 cudaError_t launch_project_fma(const MatDesc* d_mats, const int2* d_units, int32_t n_units,

@@ -39,13 +39,16 @@ struct CoeffParams {
   int32_t restore_query;
   float restore_coef;
   float* gamma_out;
-  // tensor-core path: max |C_i| of every matrix (null: not written), for the one
-  // exponent of the pass's fp16 operand scales (zo_tc_common.cuh)
-  float* amax;
+  // tensor-core path (null otherwise): the projection's operand rows [hi | lo] of the fp16 pair
+  // of C_i 2^(e_C,i), r rows of tc_hl_width(r) at matrix * r, and pinv[i] = 2^-(e_P,i),
+  // e_P,i = e_C,i + p_scale_offset(r) (zo_tc_common.cuh)
+  uint16_t* c_hl;
+  float* pinv;
 };
 
+// dependent = false: d_mats is written by work queued on the stream before this launch
 cudaError_t launch_coeff(const MatDesc* d_mats, int32_t n_mats, const CoeffParams& p,
-                         cudaStream_t s);
+                         bool dependent, cudaStream_t s);
 
 // P_i = C_i V_i^T (r x n, fp32) for the FMA weight pass.  Work units are
 // (matrix, first column) pairs of 128 columns.
@@ -121,7 +124,7 @@ cudaError_t launch_split_u(const MatDesc* d_mats, const TcMat* d_tc, const int2*
 // operand above.
 cudaError_t launch_split_u_bf16(const MatDesc* d_mats, const TcMat* d_tc, const int2* d_units,
                                 int32_t n_units, int32_t r, __nv_bfloat16* u_lin, cudaStream_t s);
-// tm_a is used for r <= 32, u_op for r >= 64; d_pinv[i] = 2^-(e_P,i) from launch_split_c.
+// tm_a is used for r <= 32, u_op for r >= 64; d_pinv[i] = 2^-(e_P,i) from launch_coeff.
 cudaError_t launch_wpass_tc(const CUtensorMap& tm_a, const void* u_op, const CUtensorMap& tm_b,
                             const CUtensorMap* d_w_maps, const TcMat* d_tc, const float* d_pinv,
                             int32_t n_mats, int64_t n_tiles, int32_t grid, int32_t r,
@@ -151,11 +154,6 @@ bool project_tc_supported(int32_t r);
 // projection units (matrix, first row)
 cudaError_t launch_split_v(const MatDesc* d_mats, const TcMat* d_tc, const int2* d_units,
                            int32_t n_units, int32_t r, uint16_t* v_hl, cudaStream_t s);
-// C_HL rows [hi | lo] of the fp16 pair of C_i 2^(e_C,i) (every pass), r rows per matrix at
-// matrix * r, with e_C,i from amax[i] = max |C_i| (the coefficient kernel's), and
-// pinv[i] = 2^-(e_P,i), e_P,i = e_C,i + p_scale_offset(r)
-cudaError_t launch_split_c(const MatDesc* d_mats, int32_t n_mats, int32_t r, const float* amax,
-                           uint16_t* c_hl, float* pinv, cudaStream_t s);
 // P_HL = [hi | lo] of the fp16 pair of (V C^T) 2^(e_P,i): tm_v over V_HL (box 64 x 128),
 // tm_c over C_HL (box 64 x r), tm_p over P_HL (box 64 x 32)
 cudaError_t launch_project_tc(const CUtensorMap& tm_v, const CUtensorMap& tm_c,

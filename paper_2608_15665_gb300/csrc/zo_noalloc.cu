@@ -157,7 +157,7 @@ extern "C" ZO_API zo_status zo_perturb_noalloc(void* W, int64_t m, int64_t n, in
   p.ca = ca;
   p.cb = cb;
   p.eps = eps;
-  e = zo::launch_coeff(d_desc, 1, p, s);
+  e = zo::launch_coeff(d_desc, 1, p, /*dependent=*/false, s);
   if (e == cudaSuccess) e = zo::launch_project_fma(d_desc, d_units, (int32_t)n_units, r, s);
   if (e == cudaSuccess) e = zo::launch_wpass_gemm(d_desc, 1, d_prefix, tiles, r, s);
   if (e != cudaSuccess) return fail(ZO_ERR_CUDA, std::string("launch: ") + cudaGetErrorString(e));

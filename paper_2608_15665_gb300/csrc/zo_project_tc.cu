@@ -31,6 +31,7 @@
 #include <cuda.h>
 
 #include "zo_kernels.h"
+#include "zo_launch.cuh"
 #include "zo_sm100.cuh"
 #include "zo_tc_common.cuh"
 
@@ -140,6 +141,8 @@ project_tc_kernel(const __grid_constant__ CUtensorMap tm_v, const __grid_constan
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = sh.tmem_base;
+  pdl_wait();
+  pdl_trigger();
 
   if (warp == 0 && lane == 0) {
     // ------------------------------------------------------------ TMA producer
@@ -359,45 +362,24 @@ project_tc_kernel(const __grid_constant__ CUtensorMap tm_v, const __grid_constan
   }
 }
 
-// Rows [hi | lo] of the scaled fp16 pair of V (units = (matrix, first row) x 128 rows, into
-// V_HL at p_row0; scale 2^kUVScaleExp) or of C (one CTA per matrix, r rows into C_HL at
-// matrix * r; scale 2^(e_C,i) from the coefficient kernel's max |C_i| = amax[i], with
-// pinv[i] = 2^-(e_P,i) written for the weight pass).  Each thread splits one row;
-// the rows are staged in shared memory with the 16-byte chunk index XOR (row & 7) and
-// written with coalesced 16-byte stores.
-template <int R, bool kC>
+// Rows [hi | lo] of the fp16 pair of V 2^kUVScaleExp (units = (matrix, first row) x 128 rows,
+// into V_HL at p_row0).  Each thread splits one row; the rows are staged in shared memory
+// with the 16-byte chunk index XOR (row & 7) and written with coalesced 16-byte stores.
+template <int R>
 __global__ void __launch_bounds__(128)
 split_rows_kernel(const MatDesc* __restrict__ mats, const TcMat* __restrict__ tcm,
-                  const int2* __restrict__ units, const float* __restrict__ amax_in,
-                  uint16_t* __restrict__ dst, float* __restrict__ pinv) {
+                  const int2* __restrict__ units, uint16_t* __restrict__ dst) {
   constexpr int kVecPerRow = 2 * R * 2 / 16;     // 16-byte chunks of [hi | lo]
   constexpr int kSw = kVecPerRow >= 8 ? 7 : kVecPerRow - 1;   // chunk swizzle within a row
-  constexpr int kStride = hl_width(R) / 8;       // chunks per row of V_HL / C_HL
+  constexpr int kStride = hl_width(R) / 8;       // chunks per row of V_HL
   extern __shared__ uint4 Os[];                  // 128 x kVecPerRow
   const int tid = threadIdx.x;
-  int i, rows;
-  int64_t row0, dst_row0;
-  const float* src;
-  if constexpr (kC) {
-    i = blockIdx.x;
-    row0 = 0;
-    rows = R;
-    src = mats[i].C;
-    dst_row0 = (int64_t)i * R;
-  } else {
-    const int2 u = units[blockIdx.x];
-    i = u.x;
-    row0 = u.y;
-    rows = (int)(mats[i].n - row0 < 128 ? mats[i].n - row0 : 128);
-    src = mats[i].V;
-    dst_row0 = (int64_t)tcm[i].p_row0 + row0;
-  }
-  float scale = exp2i(kUVScaleExp);
-  if constexpr (kC) {
-    const int e_c = coeff_scale_exp(amax_in[i]);
-    scale = exp2i(e_c);
-    if (tid == 0) pinv[i] = exp2i(-(e_c + p_scale_offset(R)));
-  }
+  const int2 u = units[blockIdx.x];
+  const int64_t row0 = u.y;
+  const int rows = (int)(mats[u.x].n - row0 < 128 ? mats[u.x].n - row0 : 128);
+  const float* src = mats[u.x].V;
+  const int64_t dst_row0 = (int64_t)tcm[u.x].p_row0 + row0;
+  const float scale = exp2i(kUVScaleExp);
   if (tid < rows) {
     const float4* s4 = reinterpret_cast<const float4*>(src + (row0 + tid) * R);
     uint4* orow = Os + tid * kVecPerRow;
@@ -430,23 +412,21 @@ cudaError_t launch_project_tc_r(const CUtensorMap& tm_v, const CUtensorMap& tm_c
   cudaError_t e = cudaFuncSetAttribute(project_tc_kernel<R, kPK>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  project_tc_kernel<R, kPK><<<grid, kProjThreads, smem, s>>>(tm_v, tm_c, tm_p, d_tc, d_units,
-                                                             n_units, d_status, kWaitCycles, p_k,
-                                                             pk_off, pinv);
-  return cudaGetLastError();
+  return launch_dependent(project_tc_kernel<R, kPK>, (unsigned)grid, kProjThreads, smem, s, 1, true,
+                          tm_v, tm_c, tm_p, d_tc, d_units, n_units, d_status, kWaitCycles, p_k,
+                          pk_off, pinv);
 }
 
-template <int R, bool kC>
+template <int R>
 cudaError_t launch_split_rows_r(const MatDesc* d_mats, const TcMat* d_tc, const int2* d_units,
-                                int32_t n_blocks, const float* amax, uint16_t* dst, float* pinv,
-                                cudaStream_t s) {
-  constexpr size_t smem = 128 * (size_t)(2 * R * 2);
+                                int32_t n_blocks, uint16_t* dst, cudaStream_t s) {
+  const size_t smem = (size_t)128 * (2 * R * 2 / 16) * sizeof(uint4);
   if (smem > 48 * 1024) {
-    cudaError_t e = cudaFuncSetAttribute(split_rows_kernel<R, kC>,
+    cudaError_t e = cudaFuncSetAttribute(split_rows_kernel<R>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
   }
-  split_rows_kernel<R, kC><<<n_blocks, 128, smem, s>>>(d_mats, d_tc, d_units, amax, dst, pinv);
+  split_rows_kernel<R><<<n_blocks, 128, smem, s>>>(d_mats, d_tc, d_units, dst);
   return cudaGetLastError();
 }
 
@@ -458,22 +438,10 @@ cudaError_t launch_split_v(const MatDesc* d_mats, const TcMat* d_tc, const int2*
                            int32_t n_units, int32_t r, uint16_t* v_hl, cudaStream_t s) {
   if (n_units <= 0) return cudaSuccess;
   switch (r) {
-    case 16: return launch_split_rows_r<16, false>(d_mats, d_tc, d_units, n_units, nullptr, v_hl, nullptr, s);
-    case 32: return launch_split_rows_r<32, false>(d_mats, d_tc, d_units, n_units, nullptr, v_hl, nullptr, s);
-    case 64: return launch_split_rows_r<64, false>(d_mats, d_tc, d_units, n_units, nullptr, v_hl, nullptr, s);
-    case 128: return launch_split_rows_r<128, false>(d_mats, d_tc, d_units, n_units, nullptr, v_hl, nullptr, s);
-    default: return cudaErrorInvalidValue;
-  }
-}
-
-cudaError_t launch_split_c(const MatDesc* d_mats, int32_t n_mats, int32_t r, const float* amax,
-                           uint16_t* c_hl, float* pinv, cudaStream_t s) {
-  if (n_mats <= 0) return cudaSuccess;
-  switch (r) {
-    case 16: return launch_split_rows_r<16, true>(d_mats, nullptr, nullptr, n_mats, amax, c_hl, pinv, s);
-    case 32: return launch_split_rows_r<32, true>(d_mats, nullptr, nullptr, n_mats, amax, c_hl, pinv, s);
-    case 64: return launch_split_rows_r<64, true>(d_mats, nullptr, nullptr, n_mats, amax, c_hl, pinv, s);
-    case 128: return launch_split_rows_r<128, true>(d_mats, nullptr, nullptr, n_mats, amax, c_hl, pinv, s);
+    case 16: return launch_split_rows_r<16>(d_mats, d_tc, d_units, n_units, v_hl, s);
+    case 32: return launch_split_rows_r<32>(d_mats, d_tc, d_units, n_units, v_hl, s);
+    case 64: return launch_split_rows_r<64>(d_mats, d_tc, d_units, n_units, v_hl, s);
+    case 128: return launch_split_rows_r<128>(d_mats, d_tc, d_units, n_units, v_hl, s);
     default: return cudaErrorInvalidValue;
   }
 }

@@ -118,8 +118,7 @@ __device__ __forceinline__ void give_up(Shared& sh, uint32_t* status) {
 // sum |U| |P|, the grade of an fp32 evaluation, at the MMA count of the bf16 pair.
 // Scales (all exact powers of two, undone in fp32 by the consumer):
 //   U, V:  2^kUVScaleExp  (|U|, |V| <= 1 for column-orthonormal bases)
-//   C_i:   2^(e_C,i) with e_C,i = 14 - E, max |C_i| < 2^E (from the maximum the coefficient
-//          kernel writes), so |C_i s| < 2^14
+//   C_i:   2^(e_C,i) with e_C,i = 14 - E, max |C_i| < 2^E (formed with C_i), so |C_i s| < 2^14
 //   P_i:   2^(e_P,i), e_P,i = e_C,i + p_scale_offset(r): |P_kj| <= ||C_k,:|| ||V_j,:|| <=
 //          sqrt(r) max |C_i|, so |P_i s| <= 2^15 (fp16 holds up to 65504)
 // The weight pass multiplies its accumulator by pinv_i 2^-kUVScaleExp, pinv_i = 2^-(e_P,i).
@@ -159,6 +158,22 @@ __device__ __forceinline__ void split8_f16(const float (&x)[8], float s, uint4& 
   }
   hi = make_uint4(hw[0], hw[1], hw[2], hw[3]);
   lo = make_uint4(lw[0], lw[1], lw[2], lw[3]);
+}
+
+// The same for 4 values.
+__device__ __forceinline__ void split4_f16(const float4& x, float s, uint2& hi, uint2& lo) {
+  const float v[4] = {x.x * s, x.y * s, x.z * s, x.w * s};
+  uint32_t hw[2], lw[2];
+#pragma unroll
+  for (int pr = 0; pr < 2; ++pr) {
+    const __half2 h2 = __floats2half2_rn(v[2 * pr], v[2 * pr + 1]);
+    const float2 hf = __half22float2(h2);
+    const __half2 l2 = __floats2half2_rn(v[2 * pr] - hf.x, v[2 * pr + 1] - hf.y);
+    hw[pr] = *reinterpret_cast<const uint32_t*>(&h2);
+    lw[pr] = *reinterpret_cast<const uint32_t*>(&l2);
+  }
+  hi = make_uint2(hw[0], hw[1]);
+  lo = make_uint2(lw[0], lw[1]);
 }
 
 // The weight-pass epilogue's arithmetic for two neighbouring bf16 weights w (packed, lower

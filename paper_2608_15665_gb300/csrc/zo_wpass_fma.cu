@@ -13,6 +13,7 @@
 #include <atomic>
 
 #include "zo_fma_common.cuh"
+#include "zo_launch.cuh"
 
 namespace zo {
 namespace {
@@ -188,6 +189,8 @@ wpass_fma_fused_kernel(const MatDesc* __restrict__ mats, int n_mats,
   const int i = find_matrix(prefix, n_mats, tile);
   const MatDesc md = mats[i];
   draw_perturb_c<R>(md, p, Cs);
+  pdl_wait();                              // the draw needs no memory
+  pdl_trigger();
   __syncthreads();
   const int64_t local = tile - md.tile0;
   if (md.dtype == 1)
@@ -214,8 +217,8 @@ template <int R>
 cudaError_t launch_fused_r(const MatDesc* d_mats, int32_t n_mats, const int64_t* d_prefix,
                            int64_t n_tiles, const CoeffParams& p, cudaStream_t s) {
   const size_t smem = sizeof(float) * (size_t)(kRows * R + R * 256 + R * R);
-  wpass_fma_fused_kernel<R><<<(unsigned)n_tiles, 256, smem, s>>>(d_mats, n_mats, d_prefix, p);
-  return cudaGetLastError();
+  return launch_dependent(wpass_fma_fused_kernel<R>, (unsigned)n_tiles, 256, smem, s, 1, true, d_mats,
+                          n_mats, d_prefix, p);
 }
 
 
@@ -226,9 +229,9 @@ cudaError_t launch_fused_r(const MatDesc* d_mats, int32_t n_mats, const int64_t*
 // chunks, and thread t updates chunks t, t + 256, ... of the tile in row-major order, so
 // a warp still reads and writes contiguous bytes of W.  The CTA forms C (drawn, or read
 // from the coefficient kernel's output) and the P columns of its tile, and stages the U
-// rows.  These sets fit in L2 and the pass is latency-bound, so a CTA puts its loads out
-// first -- U rows by cp.async straight into shared memory, then the V rows of its P
-// columns and its W chunks into registers -- and draws C while they are in flight.  The
+// rows.  These sets fit in L2 and the pass is latency-bound, so a CTA draws C while the
+// stream's previous kernel finishes, then puts all its loads out -- U rows by cp.async straight
+// into shared memory, the V rows of its P columns and its W chunks into registers.  The
 // arithmetic and its order are the tiled kernel's (P[k][c] and the update sum each by fmaf
 // from zero in ascending index, one add and one rounding into W), so both tilings give
 // bit-identical weights.
@@ -262,6 +265,10 @@ __device__ __forceinline__ void narrow_tile(const MatDesc& md, const NarrowMat& 
   const int full_end = (int)min64(chunks, md.n / VEC - ch0);  // chunks without a tail
   T* Wt = reinterpret_cast<T*>(md.W) + row0 * md.ldw + col0;
 
+  // the draw of C needs no memory: it overlaps the stream's previous kernel
+  if constexpr (kDraw) draw_perturb_c<R>(md, p, Cs);
+  pdl_wait();
+  pdl_trigger();
   // U rows of the tile: asynchronous copies into shared memory, issued first (zero-filled
   // past the last row)
   {
@@ -287,10 +294,7 @@ __device__ __forceinline__ void narrow_tile(const MatDesc& md, const NarrowMat& 
       v[j][4 * b4] = t.x; v[j][4 * b4 + 1] = t.y; v[j][4 * b4 + 2] = t.z; v[j][4 * b4 + 3] = t.w;
     }
   }
-  // C while the loads are in flight; ahead of the W loads, whose registers it would crowd
-  if constexpr (kDraw) {
-    draw_perturb_c<R>(md, p, Cs);
-  } else {
+  if constexpr (!kDraw) {
     for (int e = tid; e < R * R / 4; e += kNarrowThreads)
       reinterpret_cast<float4*>(Cs)[e] = reinterpret_cast<const float4*>(md.C)[e];
   }
@@ -400,9 +404,8 @@ cudaError_t launch_narrow_r(const MatDesc* d_mats, const NarrowMat* d_narrow,
   const int most = (int)(sizeof(float) * (R * R + R * kNarrowMaxCols + R * kNarrowChunks));
   cudaError_t e = allow_smem(wpass_narrow_kernel<R, kDraw>, most, done);
   if (e != cudaSuccess) return e;
-  wpass_narrow_kernel<R, kDraw><<<(unsigned)n_tiles, kNarrowThreads, smem, s>>>(
-      d_mats, d_narrow, d_tiles, p, (int32_t)p_floats);
-  return cudaGetLastError();
+  return launch_dependent(wpass_narrow_kernel<R, kDraw>, (unsigned)n_tiles, kNarrowThreads, smem, s, 1,
+                          true, d_mats, d_narrow, d_tiles, p, (int32_t)p_floats);
 }
 }  // namespace
 

@@ -19,6 +19,7 @@
 //    267 us against 176 and 295), elsewhere they are within 3%; 32-row tiles are slower
 //    (217 and 385 us).
 #include "zo_fma_common.cuh"
+#include "zo_launch.cuh"
 
 namespace zo {
 namespace {
@@ -191,6 +192,8 @@ wpass_gemm_kernel(const MatDesc* __restrict__ mats, int n_mats, const int64_t* _
   const int i = find_matrix(prefix, n_mats, tile);
   const MatDesc md = mats[i];
   const int64_t local = tile - __ldg(prefix + i);
+  pdl_wait();
+  pdl_trigger();
   if (md.dtype == 1)
     gemm_tile<R, __nv_bfloat16>(md, local, smem);
   else
@@ -204,8 +207,8 @@ cudaError_t launch_gemm_r(const MatDesc* d_mats, int32_t n_mats, const int64_t* 
   cudaError_t e = cudaFuncSetAttribute(wpass_gemm_kernel<R>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  wpass_gemm_kernel<R><<<(unsigned)n_tiles, kGemmThreads, smem, s>>>(d_mats, n_mats, d_prefix);
-  return cudaGetLastError();
+  return launch_dependent(wpass_gemm_kernel<R>, (unsigned)n_tiles, kGemmThreads, smem, s, 1, true,
+                          d_mats, n_mats, d_prefix);
 }
 
 }  // namespace

@@ -40,6 +40,7 @@
 #include <cuda.h>
 
 #include "zo_kernels.h"
+#include "zo_launch.cuh"
 #include "zo_cluster.cuh"
 #include "zo_sm100.cuh"
 #include "zo_tc_common.cuh"
@@ -179,6 +180,7 @@ wpass_pair_kernel(const uint4* __restrict__ u_t, const __grid_constant__ CUtenso
   cluster_sync_all();                          // both CTAs' barriers and TMEM exist
   tc_fence_after();
   const uint32_t tmem = sh.tmem_base;
+  pdl_wait();                              // (no early trigger: see zo_launch.cuh)
 
   if (warp == 0 && lane == 0) {
     // ---------------------------------------------------------------- W tiles (this CTA)
@@ -452,10 +454,9 @@ cudaError_t launch_wpass_pair(const uint4* u_t, const CUtensorMap& tm_b64,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem);
   if (e != cudaSuccess) return e;
   const long long wait = inject_wait ? kTestWaitCycles : kWaitCycles;
-  wpass_pair_kernel<<<2 * n_pairs, kThreads, kSmem, s>>>(u_t, tm_b64, d_w_maps, d_tc, d_pinv,
-                                                         n_mats, n_pair_tiles, d_status, wait,
-                                                         inject_wait ? 1 : 0);
-  return cudaGetLastError();
+  return launch_dependent(wpass_pair_kernel, 2u * n_pairs, kThreads, kSmem, s, 1, true, u_t, tm_b64,
+                          d_w_maps, d_tc, d_pinv, n_mats, n_pair_tiles, d_status, wait,
+                          inject_wait ? 1 : 0);
 }
 
 int32_t wpass_pair_max_pairs() {

@@ -35,6 +35,7 @@
 #include <cuda.h>
 
 #include "zo_kernels.h"
+#include "zo_launch.cuh"
 #include "zo_sm100.cuh"
 #include "zo_tc_common.cuh"
 
@@ -124,6 +125,7 @@ wpass_tc_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant_
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = sh.tmem_base;
+  pdl_wait();                              // (no early trigger: see zo_launch.cuh)
 
   if (warp == 0 && lane == 0) {
     // ------------------------------------------------------------ TMA producer: W tiles
@@ -363,9 +365,8 @@ cudaError_t launch_tc_r(const CUtensorMap& tm_a, const CUtensorMap& tm_b, const 
   if (e != cudaSuccess) return e;
   // with the test hook armed the wait limit is ~0.1 s so the test ends quickly
   const long long wait = inject_wait ? kTestWaitCycles : kWaitCycles;
-  wpass_tc_kernel<R><<<grid, kThreads, smem, s>>>(tm_a, tm_b, w_maps, mats, pinv, n_mats, n_tiles,
-                                                  status, wait, inject_wait ? 1 : 0);
-  return cudaGetLastError();
+  return launch_dependent(wpass_tc_kernel<R>, (unsigned)grid, kThreads, smem, s, 1, true, tm_a, tm_b,
+                          w_maps, mats, pinv, n_mats, n_tiles, status, wait, inject_wait ? 1 : 0);
 }
 
 }  // namespace

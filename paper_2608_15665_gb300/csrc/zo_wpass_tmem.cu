@@ -31,6 +31,7 @@
 #include <cuda.h>
 
 #include "zo_kernels.h"
+#include "zo_launch.cuh"
 #include "zo_sm100.cuh"
 #include "zo_tc_common.cuh"
 
@@ -128,6 +129,7 @@ wpass_tmem_kernel(const uint4* __restrict__ u_t, const __grid_constant__ CUtenso
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = sh.tmem_base;
+  pdl_wait();                              // (no early trigger: see zo_launch.cuh)
 
   if (warp == 0 && lane == 0) {
     // ------------------------------------------------------------ TMA producer: W tiles
@@ -449,10 +451,13 @@ cudaError_t launch_tmem_r(const uint4* u_t, const CUtensorMap& tm_b, const CUten
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   const long long wait = inject_wait ? kTestWaitCycles : kWaitCycles;
-  wpass_tmem_kernel<R><<<grid, TmemCfg<R>::kThreads, smem, s>>>(u_t, tm_b, w_maps, mats, pinv,
-                                                                 n_mats, n_tiles, status, wait,
-                                                                 inject_wait ? 1 : 0);
-  return cudaGetLastError();
+  // a long pass starts as one front: launched as a dependent its CTAs start apart, and the 32B
+  // set's pass (1566 tiles per CTA) took 1% longer; a 2048 x 2048 pass gains 2 of 18 us
+  const bool dependent = n_tiles <= 64 * (int64_t)grid;
+  return launch_dependent(wpass_tmem_kernel<R>, (unsigned)grid, TmemCfg<R>::kThreads, smem, s, 1,
+                          dependent,
+                          u_t, tm_b, w_maps, mats, pinv, n_mats, n_tiles, status, wait,
+                          inject_wait ? 1 : 0);
 }
 
 }  // namespace
