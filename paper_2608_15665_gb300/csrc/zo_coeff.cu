@@ -189,7 +189,7 @@ coeff_kernel(const MatDesc* __restrict__ mats, const CoeffParams p) {
   if (ctas > 1) cta2::cluster_sync_all();   // the peers have read this CTA's values
 }
 
-// P[a][j] = sum_b C[a][b] V[j][b]; one thread per column j, rows a split over ty.
+// P[a][j] = sum_b C[a][b] V[j][b], r = 4 and 8; one thread per column j, rows a split over ty.
 template <int R>
 __global__ void __launch_bounds__(256) project_fma_kernel(const MatDesc* __restrict__ mats,
                                                           const int2* __restrict__ units) {
@@ -225,17 +225,97 @@ __global__ void __launch_bounds__(256) project_fma_kernel(const MatDesc* __restr
   }
 }
 
+// The same at r = 16 ... 128 (the same terms in the same order): 128 columns by kRows rows of P
+// per CTA, a warp's lanes the columns j, j + 32, j + 64, j + 96 and its kTR rows, so that four
+// words of V and a quarter of a row's C feed 4 kTR multiply-adds (packed in pairs of columns).
+// Bound by shared-memory reads; the thread-per-column form read 16 bytes of C for 4 of them and
+// kept V's row in registers (r = 128: spilled to local memory).  V's 128 rows are transposed
+// into shared memory with an odd pitch, by 16-byte loads of eight lanes to a row, before the
+// wait: the coefficient kernel, always the stream's previous launch, triggers this one only
+// after all work before it has completed, and writes no V.
+// 12 layers of 768-wide matrices (83 K columns), the passes beside their weight kernels: 11.3 ->
+// 5.5 us at r = 32, 39 -> 24 at r = 64, 182 -> 82 at r = 128.
+template <int R>
+struct ProjectTile {
+  static constexpr int kRows = R < 64 ? R : 64;
+  static constexpr int kTR = kRows / 8;               // rows of a warp: 2, 4, 8, 8
+  static constexpr int kSplit = R / kRows;
+  static constexpr int kCols = 128, kLd = kCols + 1;
+  static constexpr size_t kSmem = sizeof(float) * (kRows * R + R * kLd);
+};
+
+template <int R>
+__global__ void __launch_bounds__(256) project_tile_kernel(const MatDesc* __restrict__ mats,
+                                                           const int2* __restrict__ units) {
+  using T = ProjectTile<R>;
+  constexpr int kLd = T::kLd, kTR = T::kTR, kCk = R < 32 ? R : 32;   // columns of V per sweep
+  extern __shared__ float4 smem4[];
+  float* Cs = reinterpret_cast<float*>(smem4);        // kRows x R
+  float* Vs = Cs + T::kRows * R;                      // R x kLd
+  const int2 u = units[blockIdx.x / T::kSplit];
+  const int a0 = blockIdx.x % T::kSplit * T::kRows;
+  const MatDesc md = mats[u.x];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+#pragma unroll 4
+  for (int w = tid; w < T::kCols * R / 4; w += 256) {
+    constexpr int kQ = kCk / 4;
+    const int k = w / (T::kCols * kQ) * kCk + 4 * (w % kQ), j = w / kQ % T::kCols;
+    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (u.y + j < md.n) v = *reinterpret_cast<const float4*>(md.V + ((int64_t)u.y + j) * R + k);
+    float* d = Vs + k * kLd + j;
+    d[0] = v.x; d[kLd] = v.y; d[2 * kLd] = v.z; d[3 * kLd] = v.w;
+  }
+  pdl_wait();
+  pdl_trigger();
+  const float4* C4 = reinterpret_cast<const float4*>(md.C + a0 * R);
+  for (int e = tid; e < T::kRows * R / 4; e += 256) smem4[e] = C4[e];
+  __syncthreads();
+  float2 acc[kTR][2];
+#pragma unroll
+  for (int i = 0; i < kTR; ++i) acc[i][0] = acc[i][1] = make_float2(0.f, 0.f);
+  const float* c = Cs + warp * kTR * R;
+#pragma unroll 2
+  for (int k4 = 0; k4 < R; k4 += 4) {
+    float4 cv[kTR];
+#pragma unroll
+    for (int i = 0; i < kTR; ++i) cv[i] = *reinterpret_cast<const float4*>(c + i * R + k4);
+#pragma unroll
+    for (int kk = 0; kk < 4; ++kk) {
+      const float* v = Vs + (k4 + kk) * kLd + lane;
+      const float2 v0 = make_float2(v[0], v[32]), v1 = make_float2(v[64], v[96]);
+#pragma unroll
+      for (int i = 0; i < kTR; ++i) {
+        const float x = kk == 0 ? cv[i].x : kk == 1 ? cv[i].y : kk == 2 ? cv[i].z : cv[i].w;
+        acc[i][0] = fma2(make_float2(x, x), v0, acc[i][0]);
+        acc[i][1] = fma2(make_float2(x, x), v1, acc[i][1]);
+      }
+    }
+  }
+  const int64_t j = (int64_t)u.y + lane;
+#pragma unroll
+  for (int i = 0; i < kTR; ++i) {
+    float* p = md.P + (int64_t)(a0 + warp * kTR + i) * md.n;
+    if (j < md.n) p[j] = acc[i][0].x;
+    if (j + 32 < md.n) p[j + 32] = acc[i][0].y;
+    if (j + 64 < md.n) p[j + 64] = acc[i][1].x;
+    if (j + 96 < md.n) p[j + 96] = acc[i][1].y;
+  }
+}
+
 template <int R>
 cudaError_t launch_project_fma_r(const MatDesc* d_mats, const int2* d_units, int32_t n_units,
                                  cudaStream_t s) {
-  const size_t smem = sizeof(float) * R * R;
-  if (smem > 48 * 1024) {
-    cudaError_t e = cudaFuncSetAttribute(project_fma_kernel<R>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if constexpr (R >= 16) {
+    using T = ProjectTile<R>;
+    const cudaError_t e = cudaFuncSetAttribute(
+        project_tile_kernel<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)T::kSmem);
     if (e != cudaSuccess) return e;
+    return launch_dependent(project_tile_kernel<R>, (unsigned)n_units * T::kSplit, 256, T::kSmem,
+                            s, 1, true, d_mats, d_units);
+  } else {
+    return launch_dependent(project_fma_kernel<R>, (unsigned)n_units, 256, sizeof(float) * R * R, s,
+                            1, true, d_mats, d_units);
   }
-  return launch_dependent(project_fma_kernel<R>, (unsigned)n_units, 256, smem, s, 1, true, d_mats,
-                          d_units);
 }
 
 }  // namespace
