@@ -715,12 +715,11 @@ zo_status zo_create(zo_ctx** out, const zo_matrix* mats, int32_t n_mats, int32_t
   int64_t off = 0;
   std::vector<zo::CqPanel> cq_panels;
   std::vector<zo::CqChunk> cq_chunks;
-  const int64_t chunk_rows = zo::cq_chunk_rows(r);
   auto add_cholqr = [&](float* out, int64_t rows, uint32_t gidx, uint32_t tag) {
     zo::CqPanel p{out, rows, gidx, tag, (int32_t)cq_chunks.size(), 0};
-    for (int64_t r0 = 0; r0 < rows; r0 += chunk_rows) {
+    for (int64_t r0 = 0; r0 < rows; r0 += zo::kCqChunkRows) {
       cq_chunks.push_back({r0, (int32_t)cq_panels.size(),
-                           (int32_t)std::min<int64_t>(chunk_rows, rows - r0)});
+                           (int32_t)std::min<int64_t>(zo::kCqChunkRows, rows - r0)});
       ++p.n_chunks;
     }
     cq_panels.push_back(p);

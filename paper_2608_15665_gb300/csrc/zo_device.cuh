@@ -80,6 +80,11 @@ __device__ __forceinline__ uint4 philox4x32_10(uint4 c, uint32_t k0, uint32_t k1
   return c;
 }
 
+// u = ((x >> 8) + 1) * 2^-24 in (0, 1]; the integer fits 24 bits, so exact in fp32.
+__device__ __forceinline__ float u01(uint32_t x) {
+  return __uint2float_rn((x >> 8) + 1u) * 5.9604644775390625e-08f;
+}
+
 // The transform below runs on one value at a time (float) or on packed pairs (float2); both
 // round every operation alike, so they give the same bits.
 __device__ __forceinline__ float vfma(float a, float b, float c) { return fmaf(a, b, c); }
@@ -203,21 +208,15 @@ __device__ __forceinline__ void box_muller_parts(const uint32_t (&xa)[kV * Lanes
   }
 }
 
-// One pair of words.
+// The same of one pair of words by CUDA's functions: what forms Z and bf16 weights' Omega, which
+// are few (the transform above is for the full-space pass's draws and fp32 bases).  The two
+// differ in the last place, and bf16 weights at a rounding boundary show it: up to rel 1.3e-5
+// of a 1 M-weight set after a step.
 __device__ __forceinline__ float2 box_muller(uint32_t xa, uint32_t xb) {
-  const uint32_t a[1] = {xa}, b[1] = {xb};
-  float nr[1], c[1], s[1];
-  box_muller_parts<1, float>(a, b, nr, c, s);
-  return make_float2(__fmul_rn(nr[0], c[0]), __fmul_rn(nr[0], s[0]));
-}
-// The four words of a counter, in packed arithmetic.
-__device__ __forceinline__ float4 box_muller4(uint4 x) {
-  const uint32_t a[2] = {x.x, x.z}, b[2] = {x.y, x.w};
-  float2 nr[1], c[1], s[1];
-  box_muller_parts<1, float2>(a, b, nr, c, s);
-  c[0] = mul2(nr[0], c[0]);
-  s[0] = mul2(nr[0], s[0]);
-  return make_float4(c[0].x, s[0].x, c[0].y, s[0].y);
+  const float rad = sqrtf(-2.0f * logf(u01(xa)));
+  float s, c;
+  sincospif(2.0f * u01(xb), &s, &c);
+  return make_float2(rad * c, rad * s);
 }
 
 // Four normals of counter word `c4` of the stream (seed, x1, x2, x3).
@@ -225,7 +224,20 @@ __device__ __forceinline__ float4 normal4(uint64_t seed, uint32_t c4, uint32_t x
                                           uint32_t x3) {
   const uint4 w = philox4x32_10(make_uint4(c4, x1, x2, x3), static_cast<uint32_t>(seed),
                                 static_cast<uint32_t>(seed >> 32));
-  return box_muller4(w);
+  const float2 a = box_muller(w.x, w.y);
+  const float2 b = box_muller(w.z, w.w);
+  return make_float4(a.x, a.y, b.x, b.y);
+}
+__device__ __forceinline__ float4 normal4_packed(uint64_t seed, uint32_t c4, uint32_t x1,
+                                                 uint32_t x2, uint32_t x3) {
+  const uint4 w = philox4x32_10(make_uint4(c4, x1, x2, x3), static_cast<uint32_t>(seed),
+                                static_cast<uint32_t>(seed >> 32));
+  const uint32_t a[2] = {w.x, w.z}, b[2] = {w.y, w.w};
+  float2 nr[1], c[1], s[1];
+  box_muller_parts<1, float2>(a, b, nr, c, s);
+  c[0] = mul2(nr[0], c[0]);
+  s[0] = mul2(nr[0], s[0]);
+  return make_float4(c[0].x, s[0].x, c[0].y, s[0].y);
 }
 
 // ---------------------------------------------------------------------------

@@ -271,9 +271,7 @@ cudaError_t launch_linear_few(const CUtensorMap& tm_x, const CUtensorMap& tm_xs,
                               cudaStream_t s);
 
 // ---- refresh of tall panels at r = 16 ... 128: CholeskyQR2 (zo_cholqr.cu) ----------
-// rows per partial Gram matrix: by r alone, so that a panel's bits do not depend on the others.
-// (At r = 16 and 32 a thread's part of 512 rows was as short as its sums' exchange.)
-constexpr int32_t cq_chunk_rows(int32_t r) { return r <= 32 ? 1024 : 512; }
+constexpr int32_t kCqChunkRows = 1024;   // rows per partial Gram matrix
 struct CqPanel {
   float* out;          // U_i or V_i: rows x r, row-major; receives Q
   int64_t rows;
@@ -285,7 +283,7 @@ struct CqPanel {
 struct CqChunk {
   int64_t row0;        // first panel row of the chunk
   int32_t panel;
-  int32_t nrows;       // <= cq_chunk_rows(r)
+  int32_t nrows;       // <= kCqChunkRows
 };
 bool cholqr_supported(int32_t r);
 // Six launches: Gram, Cholesky + inverse, apply; twice.  d_partial: n_chunks x r x r

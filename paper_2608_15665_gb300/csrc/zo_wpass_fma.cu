@@ -149,26 +149,21 @@ __device__ __forceinline__ void wpass_tile(const MatDesc& md, int64_t local, flo
 
 // C = eps (ca Z_qa + cb Z_qb) of one matrix into shared memory, with the coefficient
 // kernel's arithmetic (so that every path forms the same C).  One thread per pair of
-// elements: the pass waits for this chain, so the pair's Z_qa and Z_qb go through one packed
-// transform and R^2 / 2 threads (at most a warp) run it once.
+// elements: the pass waits for this chain, so R^2 / 2 threads (at most a warp) run it once.
 template <int R>
 __device__ __forceinline__ void draw_perturb_c(const MatDesc& md, const CoeffParams& p, float* Cs) {
   for (int e = threadIdx.x; e < R * R / 2; e += blockDim.x) {
     const uint32_t lo = (uint32_t)p.seed, hi = (uint32_t)(p.seed >> 32);
     const uint32_t c = (uint32_t)e >> 1;
-    const uint4 wa = philox4x32_10(make_uint4(c, md.gidx, p.t, query_word(kTagZ, (uint32_t)p.qa)), lo, hi);
-    uint4 wb = wa;
-    if (p.qb >= 0)
-      wb = philox4x32_10(make_uint4(c, md.gidx, p.t, query_word(kTagZ, (uint32_t)p.qb)), lo, hi);
     const bool odd = e & 1;
-    const uint32_t xa[2] = {odd ? wa.z : wa.x, odd ? wb.z : wb.x};
-    const uint32_t xb[2] = {odd ? wa.w : wa.y, odd ? wb.w : wb.y};
-    float2 nr[1], cs[1], sn[1];
-    box_muller_parts<1, float2>(xa, xb, nr, cs, sn);
-    float2 acc = make_float2(p.ca * __fmul_rn(nr[0].x, cs[0].x), p.ca * __fmul_rn(nr[0].x, sn[0].x));
-    if (p.qb >= 0)
-      acc = make_float2(fmaf(p.cb, __fmul_rn(nr[0].y, cs[0].y), acc.x),
-                        fmaf(p.cb, __fmul_rn(nr[0].y, sn[0].y), acc.y));
+    const uint4 wa = philox4x32_10(make_uint4(c, md.gidx, p.t, query_word(kTagZ, (uint32_t)p.qa)), lo, hi);
+    const float2 za = box_muller(odd ? wa.z : wa.x, odd ? wa.w : wa.y);
+    float2 acc = make_float2(p.ca * za.x, p.ca * za.y);
+    if (p.qb >= 0) {
+      const uint4 wb = philox4x32_10(make_uint4(c, md.gidx, p.t, query_word(kTagZ, (uint32_t)p.qb)), lo, hi);
+      const float2 zb = box_muller(odd ? wb.z : wb.x, odd ? wb.w : wb.y);
+      acc = make_float2(fmaf(p.cb, zb.x, acc.x), fmaf(p.cb, zb.y, acc.y));
+    }
     reinterpret_cast<float2*>(Cs)[e] = make_float2(p.eps * acc.x, p.eps * acc.y);
   }
 }
