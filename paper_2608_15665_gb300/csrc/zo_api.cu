@@ -695,15 +695,18 @@ zo_status zo_create(zo_ctx** out, const zo_matrix* mats, int32_t n_mats, int32_t
   int64_t qr_floats = 0;
   // a panel with rows >= 4r has kappa(Omega) <= ~3, well inside CholeskyQR2's range
   auto use_cholqr = [&](int64_t rows) { return zo::cholqr_supported(r) && rows >= 4 * (int64_t)r; };
-  auto use_small = [&](int64_t rows) {
-    return zo::cholqr_small_short(r, rows) || zo::cholqr_small_ctas(r, rows) > 0;
+  // Bases of bf16 weights at r = 4 and 8 keep the TSQR's bits: bases that differ in the last
+  // place move a pass's few weights at a rounding boundary by a whole bf16 unit (up to rel
+  // 2.3e-5 of a 350 K-weight set after a step; fp32 weights: 2e-8).
+  auto use_small = [&](int64_t rows, int32_t dtype) {
+    return dtype == 0 && (zo::cholqr_small_short(r, rows) || zo::cholqr_small_ctas(r, rows) > 0);
   };
-  auto use_tsqr = [&](int64_t rows) { return !use_cholqr(rows) && !use_small(rows); };
+  auto use_tsqr = [&](int64_t rows, int32_t dtype) { return !use_cholqr(rows) && !use_small(rows, dtype); };
   {
     std::vector<QrLevel> dry;
     for (int32_t i = 0; i < n_mats; ++i) {
-      if (use_tsqr(mats[i].m)) plan_panel(nullptr, mats[i].m, r, 0, zo::kTagOmegaU, B, dry, nullptr, &qr_floats);
-      if (use_tsqr(mats[i].n)) plan_panel(nullptr, mats[i].n, r, 0, zo::kTagOmegaV, B, dry, nullptr, &qr_floats);
+      if (use_tsqr(mats[i].m, mats[i].dtype)) plan_panel(nullptr, mats[i].m, r, 0, zo::kTagOmegaU, B, dry, nullptr, &qr_floats);
+      if (use_tsqr(mats[i].n, mats[i].dtype)) plan_panel(nullptr, mats[i].n, r, 0, zo::kTagOmegaV, B, dry, nullptr, &qr_floats);
     }
   }
   e = cudaMalloc(&c->d_qr_ws, sizeof(float) * std::max<int64_t>(qr_floats, 4));
@@ -725,10 +728,10 @@ zo_status zo_create(zo_ctx** out, const zo_matrix* mats, int32_t n_mats, int32_t
     cq_panels.push_back(p);
   };
   std::vector<zo::CqPanel> small[5];     // short ones, then tall ones of 1, 2, 4, 8 CTAs
-  auto add_panel = [&](float* out, int64_t rows, uint32_t gidx, uint32_t tag) {
+  auto add_panel = [&](float* out, int64_t rows, int32_t dtype, uint32_t gidx, uint32_t tag) {
     if (use_cholqr(rows)) {
       add_cholqr(out, rows, gidx, tag);
-    } else if (use_small(rows)) {
+    } else if (use_small(rows, dtype)) {
       const int32_t ctas = zo::cholqr_small_ctas(r, rows);
       small[ctas == 0 ? 0 : ctas == 1 ? 1 : ctas == 2 ? 2 : ctas == 4 ? 3 : 4].push_back(
           {out, rows, gidx, tag, 0, 0});
@@ -738,8 +741,8 @@ zo_status zo_create(zo_ctx** out, const zo_matrix* mats, int32_t n_mats, int32_t
   };
   for (int32_t i = 0; i < n_mats; ++i) {
     const uint32_t gidx = matrix_index_base + (uint32_t)i;
-    add_panel(mats[i].U, mats[i].m, gidx, zo::kTagOmegaU);
-    add_panel(mats[i].V, mats[i].n, gidx, zo::kTagOmegaV);
+    add_panel(mats[i].U, mats[i].m, mats[i].dtype, gidx, zo::kTagOmegaU);
+    add_panel(mats[i].V, mats[i].n, mats[i].dtype, gidx, zo::kTagOmegaV);
   }
   std::vector<zo::CqPanel> small_panels;
   for (const auto& v : small) small_panels.insert(small_panels.end(), v.begin(), v.end());

@@ -17,18 +17,21 @@
 // exactly as the TSQR of zo_qr.cu draws it; panels shorter than 4r keep the TSQR.
 //
 // Launches per refresh: gram(Omega, which also writes Omega to the panel), chol,
-// apply(Omega -> Q1), gram(Q1), chol, apply(Q1 -> Q).  Sums over rows are fixed-order (groups
-// of threads within a chunk of rows, then chunk by chunk), so a refresh is bit-reproducible.
+// apply(Omega -> Q1), gram(Q1), chol, apply(Q1 -> Q).  Every sum is one chain of fp32
+// multiply-adds in a fixed order (a Gram element over the rows of a 1024-row chunk, then chunk by
+// chunk; a factor's and a product's elements over their index), whatever the tiles: a refresh is
+// bit-reproducible, whichever matrices share the context.  The tiles keep the chains because
+// bf16 weights show them: with the rows of a chunk dealt to groups of threads (Q's error against
+// 64 bits halves, 32B set 1.67 ms) a step of a 1 M-weight set moved by up to rel 1.3e-5.
 //
 // Bound: fp32 multiply-adds (8 r^2 per row over the four products, 5.3 r^2 with the triangles
-// left out) and Omega's draws; at r = 128 on few panels the factorisations.  So: 8 x 8 (Gram)
-// and up to 8 x 8 (apply) register tiles in packed multiply-adds, which shared memory can
-// feed; only the Gram matrix's lower 8 x 8 blocks, the rows of a chunk dealt to as many groups
-// of threads as the blocks leave room for; only L^-1's lower half where a thread's columns
-// allow; Omega drawn once; and a blocked Cholesky.
-// Refresh of 16 layers of the 32B set at r = 64: 2.64 -> 1.67 ms; of 32 of the 7B set at r = 32:
-// 1.29 -> 0.81; of one at r = 128: 1.55 -> 0.44.  Q's error against 64 bits is 0.4 to 0.7 of
-// the former kernels' (shorter chains of sums).
+// left out) and Omega's draws; at r = 128 on few panels the factorisations.  So: register tiles
+// in packed multiply-adds, which shared memory can feed; only the Gram matrix's lower blocks;
+// only L^-1's lower half where a thread's columns allow; Omega drawn once; and a blocked
+// Cholesky.
+// Refresh of 16 layers of the 32B set at r = 64: 2.64 -> 1.91 ms; of 32 of the 7B set at r = 32:
+// 1.29 -> 0.93, of one 0.191 -> 0.141; of 8 at r = 128: 4.38 -> 1.88; of 24 of the 1.3B set at
+// r = 16: 0.278 -> 0.204.
 #include "zo_cluster.cuh"
 #include "zo_fma_common.cuh"
 #include "zo_kernels.h"
@@ -39,57 +42,97 @@ namespace {
 
 using namespace fma;
 
-// ---------------------------------------------------------------- Gram matrix of a chunk
-// 8 x 8 blocks of the lower triangle, a block of kGroups threads, which take the chunk's rows
-// in turn.  Lanes of a warp read neighbouring rows of the same columns: with a row pitch of
-// R + 4 floats no two of a load's 16-byte words share banks.  Rows pass through a ring of
-// stages, copied two ahead (one ahead left the copies' latency exposed) or drawn one ahead.
-// Bound by shared-memory reads and multiply-adds together: 4 16-byte loads per 32 packed
-// multiply-adds, either 34 us of the 75 that 4 layers of the 32B set take at r = 64 (the bytes:
-// 20); on Omega by its draws (another 59 us).
-template <int R, bool kOmega>
+// ---------------------------------------------------------------- Gram matrices of chunks
+// A CTA takes kG chunks; of each, T x T blocks of the lower triangle, a block per thread.  Every
+// element is one chain of fp32 multiply-adds over the chunk's rows in order, whatever the tile,
+// so the tile may follow the set: 8 x 8 at r = 64 and 128, where shared memory must feed the
+// multiply-adds; smaller ones, and one chunk per CTA, where chains are what is short.  256
+// threads load or draw a stage even where fewer multiply (one 7B layer at r = 32, CTAs of the
+// 64 that multiply: 205 us a refresh; of 256: 141).  Rows pass through a ring of stages, copied
+// two ahead or drawn one ahead.
+//
+// 4 layers of the 32B set at r = 64: 93 us (4 x 4 tiles, 512 chunks), where the bytes take 20 and
+// an 8 x 8 tile's multiply-adds and its shared-memory reads 34 each; Omega's draws add 63.
+template <int R, int T, int kG, bool kOmega>
 struct Gram {
-  static constexpr int kBlocks = (R / 8) * (R / 8 + 1) / 2;           // 3, 10, 36, 136
-  static constexpr int kGroups = R == 16 ? 96 : R == 32 ? 32 : R == 64 ? 8 : 2;
-  static constexpr int kThreads = (kBlocks * kGroups + 31) / 32 * 32;           // 288; 320 at R = 32
-  static constexpr int kSub = R == 16 ? 384 : R == 32 ? 192 : R == 64 ? 64 : 32;   // rows of a stage
+  static constexpr int kN = R / T;
+  static constexpr int kBlocks = kN * (kN + 1) / 2;
+  static constexpr int kBlockThreads = (kBlocks * kG + 31) / 32 * 32;
+  static constexpr int kThreads = kBlockThreads > 256 ? kBlockThreads : 256;
+  static constexpr int kPer = 256 / kG;                               // loading threads of a chunk
+  static constexpr int kSub = kG > 4 ? 16 : kG > 1 ? 32 : R == 16 ? 128 : R == 32 ? 64 : 32;
   static constexpr int kStages = kOmega ? 2 : 3;
   static constexpr int kLd = R + 4;
-  static constexpr int kStage = kSub * kLd;                           // floats
+  static constexpr int kStage = kG * kSub * kLd;                      // floats
   static constexpr size_t kSmem = sizeof(float) * kStages * kStage;
+  static_assert(kSub * R / 4 % kPer == 0, "whole words per loading thread");
 };
 
-template <int R, bool kOmega>
-__global__ void __launch_bounds__(Gram<R, kOmega>::kThreads, 2)
-cq_gram_kernel(const CqPanel* __restrict__ panels, const CqChunk* __restrict__ chunks,
+// T consecutive floats as pairs
+template <int T>
+__device__ __forceinline__ void load_pairs(const float* p, float2 (&v)[T / 2]) {
+  if constexpr (T == 2) {
+    v[0] = *reinterpret_cast<const float2*>(p);
+  } else {
+#pragma unroll
+    for (int q = 0; q < T / 4; ++q) {
+      const float4 x = reinterpret_cast<const float4*>(p)[q];
+      v[2 * q] = make_float2(x.x, x.y);
+      v[2 * q + 1] = make_float2(x.z, x.w);
+    }
+  }
+}
+
+template <int R, int T, int kG, bool kOmega>
+__global__ void __launch_bounds__(Gram<R, T, kG, kOmega>::kThreads)
+cq_gram_kernel(const CqPanel* __restrict__ panels, const CqChunk* __restrict__ chunks, int n_chunks,
                float* __restrict__ partial, uint64_t seed, uint32_t refresh_idx) {
-  using Cfg = Gram<R, kOmega>;
-  constexpr int kLd = Cfg::kLd, kW = R / 4, kG = Cfg::kGroups, kStages = Cfg::kStages;
+  using Cfg = Gram<R, T, kG, kOmega>;
+  constexpr int kLd = Cfg::kLd, kW = R / 4, kStages = Cfg::kStages, kSub = Cfg::kSub, kP = T / 2;
   extern __shared__ __align__(16) float cq_smem[];
-  const CqChunk ch = chunks[blockIdx.x];
-  const CqPanel pn = panels[ch.panel];
-  const int tid = threadIdx.x, lane = tid & 31;
-  const int g = tid % kG, u = min(tid / kG, Cfg::kBlocks - 1);
+  __shared__ int rows[kG];
+  const int tid = threadIdx.x, chunk0 = blockIdx.x * kG;
+  // thread's chunk to load: 256 threads, kPer for each
+  const int q = min(tid / Cfg::kPer, kG - 1), w0 = tid % Cfg::kPer;
+  float* src = nullptr;                          // the chunk's rows in its panel
+  int words = 0;                                 // 4-float words in them
+  uint32_t c0 = 0, gidx = 0, tag = 0;            // the first one's counter; the stream
+  if (tid < 256 && chunk0 + q < n_chunks) {
+    const CqChunk ch = chunks[chunk0 + q];
+    const CqPanel pn = panels[ch.panel];
+    src = pn.out + ch.row0 * R;
+    words = ch.nrows * kW;
+    c0 = (uint32_t)((ch.row0 * R) >> 2);
+    gidx = pn.gidx;
+    tag = query_word(pn.tag, 0);
+  }
+  if (w0 == 0 && tid < 256) rows[q] = words / kW;
+  __syncthreads();
+  const int g = min(tid / Cfg::kBlocks, kG - 1), u = tid % Cfg::kBlocks;
   int bi = 0;
   while ((bi + 1) * (bi + 2) / 2 <= u) ++bi;
-  const int bj = u - bi * (bi + 1) / 2;                               // bj <= bi
-  const int n_sub = (ch.nrows + Cfg::kSub - 1) / Cfg::kSub;
+  const int bj = u - bi * (bi + 1) / 2;          // bj <= bi
+  const bool mine = tid < Cfg::kBlocks * kG;
+  int most = 0;
+#pragma unroll
+  for (int i = 0; i < kG; ++i) most = max(most, rows[i]);
+  const int n_sub = (most + kSub - 1) / kSub;
 
   // stage t's rows: drawn (and kept in the panel), or copied
   auto stage = [&](int t) {
     if (t < n_sub) {
-      const int s0 = t * Cfg::kSub, n = min(Cfg::kSub, ch.nrows - s0);
-      float* dst = cq_smem + t % kStages * Cfg::kStage;
-      float* src = pn.out + (ch.row0 + s0) * R;
-      for (int w = tid; w < n * kW; w += Cfg::kThreads) {
+      float* dst = cq_smem + t % kStages * Cfg::kStage + q * kSub * kLd;
+#pragma unroll
+      for (int i = 0; i < kSub * kW / Cfg::kPer; ++i) {
+        const int w = w0 + i * Cfg::kPer, v = t * kSub * kW + w;
+        if (v >= words) continue;
         float* d = dst + w / kW * kLd + 4 * (w % kW);
         if constexpr (kOmega) {
-          const uint32_t c = (uint32_t)((((ch.row0 + s0) * R) >> 2) + w);
-          const float4 z = normal4(seed, c, pn.gidx, refresh_idx, query_word(pn.tag, 0));
-          *reinterpret_cast<float4*>(src + 4 * w) = z;
+          const float4 z = normal4(seed, c0 + (uint32_t)v, gidx, refresh_idx, tag);
+          *reinterpret_cast<float4*>(src + 4 * v) = z;
           *reinterpret_cast<float4*>(d) = z;
         } else {
-          cp_async_16(d, src + 4 * w, 16);
+          cp_async_16(d, src + 4 * v, 16);
         }
       }
     }
@@ -98,82 +141,57 @@ cq_gram_kernel(const CqPanel* __restrict__ panels, const CqChunk* __restrict__ c
 
   // acc[e][a][b]: columns 2b, 2b + 1 of the block with rows 2a, 2a + 1 (e = 0) or 2a + 1, 2a
   // (e = 1): swapped pairs take half the register moves of duplicated operands
-  float2 acc[2][4][4];
+  float2 acc[2][kP][kP];
 #pragma unroll
-  for (int e = 0; e < 32; ++e) acc[e / 16][e / 4 % 4][e % 4] = make_float2(0.f, 0.f);
+  for (int e = 0; e < 2 * kP * kP; ++e)
+    acc[e / (kP * kP)][e / kP % kP][e % kP] = make_float2(0.f, 0.f);
 #pragma unroll
   for (int t = 0; t < kStages - 1; ++t) stage(t);
   for (int t = 0; t < n_sub; ++t) {
     if constexpr (!kOmega) cp_async_wait<kStages - 2>();
     __syncthreads();                             // stage t is there, stage t - 1 is read
     stage(t + kStages - 1);
-    const int n = min(Cfg::kSub, ch.nrows - t * Cfg::kSub);
-    const float* X = cq_smem + t % kStages * Cfg::kStage;
-#pragma unroll 2
-    for (int k = g; k < n; k += kG) {
-      const float4* xi = reinterpret_cast<const float4*>(X + k * kLd + 8 * bi);
-      const float4* xj = reinterpret_cast<const float4*>(X + k * kLd + 8 * bj);
-      const float4 i0 = xi[0], i1 = xi[1], j0 = xj[0], j1 = xj[1];
-      const float2 a4[4] = {make_float2(i0.x, i0.y), make_float2(i0.z, i0.w),
-                            make_float2(i1.x, i1.y), make_float2(i1.z, i1.w)};
-      const float2 b4[4] = {make_float2(j0.x, j0.y), make_float2(j0.z, j0.w),
-                            make_float2(j1.x, j1.y), make_float2(j1.z, j1.w)};
+    if (!mine) continue;
+    const int n = min(kSub, rows[g] - t * kSub);
+    const float* X = cq_smem + t % kStages * Cfg::kStage + g * kSub * kLd;
+#pragma unroll (T == 8 ? 2 : 4)
+    for (int k = 0; k < n; ++k) {
+      float2 a2[kP], b2[kP];
+      load_pairs<T>(X + k * kLd + T * bi, a2);
+      load_pairs<T>(X + k * kLd + T * bj, b2);
 #pragma unroll
-      for (int a = 0; a < 4; ++a) {
-        const float2 sw = make_float2(a4[a].y, a4[a].x);
+      for (int a = 0; a < kP; ++a) {
+        const float2 sw = make_float2(a2[a].y, a2[a].x);
 #pragma unroll
-        for (int b = 0; b < 4; ++b) {
-          acc[0][a][b] = fma2(a4[a], b4[b], acc[0][a][b]);
-          acc[1][a][b] = fma2(sw, b4[b], acc[1][a][b]);
+        for (int b = 0; b < kP; ++b) {
+          acc[0][a][b] = fma2(a2[a], b2[b], acc[0][a][b]);
+          acc[1][a][b] = fma2(sw, b2[b], acc[1][a][b]);
         }
       }
     }
   }
-  // The groups' sums, by halves: a lane hands the other half of its elements to its partner and
-  // adds the partner's to its own, so it ends with the kKeep elements from kKeep (lane % kW2).
-  constexpr int kW2 = kG < 32 ? kG : 32, kKeep = 64 / kW2;
-  float v[64];
+  if (!mine || rows[g] == 0) return;
+  float* out = partial + (int64_t)(chunk0 + g) * R * R + T * bi * R + T * bj;
 #pragma unroll
-  for (int e = 0; e < 16; ++e) {
-    const int a = e / 4, b = e % 4;
-    v[16 * a + 2 * b] = acc[0][a][b].x;
-    v[16 * a + 2 * b + 1] = acc[1][a][b].y;
-    v[16 * a + 8 + 2 * b] = acc[1][a][b].x;
-    v[16 * a + 8 + 2 * b + 1] = acc[0][a][b].y;
-  }
+  for (int a = 0; a < kP; ++a)
 #pragma unroll
-  for (int off = kW2 / 2; off > 0; off /= 2) {
-    const int n = off * kKeep;
-    const bool up = lane & off;
-#pragma unroll
-    for (int i = 0; i < n; ++i) {
-      const float send = up ? v[i] : v[i + n], keep = up ? v[i + n] : v[i];
-      v[i] = keep + __shfl_xor_sync(0xffffffffu, send, off);
+    for (int b = 0; b < kP; ++b) {
+      const float2 d = acc[0][a][b], x = acc[1][a][b];
+      *reinterpret_cast<float2*>(out + 2 * a * R + 2 * b) = make_float2(d.x, x.y);
+      *reinterpret_cast<float2*>(out + (2 * a + 1) * R + 2 * b) = make_float2(x.x, d.y);
     }
-  }
-  const int m = kKeep * (lane % kW2);
-  if constexpr (kG > 32) {                       // R = 16: a block is three warps' (kKeep = 2)
-    __syncthreads();
-    const int warp = tid / 32;
-    if (warp % 3 > 0) *reinterpret_cast<float2*>(cq_smem + 64 * warp + m) = make_float2(v[0], v[1]);
-    __syncthreads();
-    if (warp % 3 > 0) return;
-#pragma unroll
-    for (int q = 1; q < 3; ++q) {
-      const float2 o = *reinterpret_cast<const float2*>(cq_smem + 64 * (warp + q) + m);
-      v[0] += o.x;
-      v[1] += o.y;
-    }
-  }
-  if (tid / kG >= Cfg::kBlocks) return;
-  float* out = partial + (int64_t)blockIdx.x * R * R + (8 * bi + m / 8) * R + 8 * bj + m % 8;
-  if constexpr (kKeep == 2) {
-    *reinterpret_cast<float2*>(out) = make_float2(v[0], v[1]);
-  } else {
-#pragma unroll
-    for (int q = 0; q < kKeep; q += 4)
-      *reinterpret_cast<float4*>(out + q / 8 * R + q % 8) = make_float4(v[q], v[q + 1], v[q + 2], v[q + 3]);
-  }
+}
+
+template <int R, int T, int kG, bool kOmega>
+cudaError_t launch_gram(const CqPanel* d_panels, const CqChunk* d_chunks, int32_t n_chunks,
+                        float* d_partial, uint64_t seed, uint32_t refresh_idx, cudaStream_t s) {
+  using Cfg = Gram<R, T, kG, kOmega>;
+  const cudaError_t e = cudaFuncSetAttribute(
+      cq_gram_kernel<R, T, kG, kOmega>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg::kSmem);
+  if (e != cudaSuccess) return e;
+  cq_gram_kernel<R, T, kG, kOmega><<<(n_chunks + kG - 1) / kG, Cfg::kThreads, Cfg::kSmem, s>>>(
+      d_panels, d_chunks, n_chunks, d_partial, seed, refresh_idx);
+  return cudaGetLastError();
 }
 
 // ---------------------------------------------------------------- Cholesky factor, inverse
@@ -184,14 +202,14 @@ cq_gram_kernel(const CqPanel* __restrict__ panels, const CqChunk* __restrict__ c
 // non-positive pivot -- not expected for a tall Gaussian panel -- sets kDevNotPosDef and leaves
 // L^-1 = 0.
 //
-// Latency-bound: a block's columns are one warp's registers, so that the CTA synchronises 4
+// Latency-bound: a block's columns are one warp's registers, so that the CTA synchronises 3
 // times per 16 columns instead of 3 times per column, and the products around them, those of
-// the inverse among them, run on all threads.  56 panels at r = 128: 440 -> 64 us; at r = 64:
-// 113 -> 28 us.  (One CTA per panel: 106 and 52.)
+// the inverse among them, run on all threads.  56 panels at r = 128: 440 -> 78 us; at r = 64:
+// 113 -> 32 us (the inverse's divisions, part of its chains, are 10 of the 78).
 constexpr int kCholCtas = 4;
 constexpr int kNb = 16;
 template <int R>
-constexpr int kCholThreads = R == 128 ? 512 : 256;   // >= 4 (R - kNb): phase 2, one item each
+constexpr int kCholThreads = R == 128 ? 512 : 256;   // >= R: phase 2
 
 template <int R>
 __global__ void __launch_bounds__(kCholThreads<R>)
@@ -202,6 +220,7 @@ cq_chol_kernel(const CqPanel* __restrict__ panels, const float* __restrict__ par
   // R x kLd: G, whose lower triangle becomes L below its diagonal blocks; the transpose of L^-1
   // (on the way, of the L L^-1 of rows to come) in the diagonal blocks and above
   float* A = cq_smem;
+  __shared__ float LT[kNb][kNb], diag[kNb], dinv[kNb];   // LT[j][i] = L[k0 + i][k0 + j]
   __shared__ int bad;
   const CqPanel pn = panels[blockIdx.x / kCholCtas];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -235,8 +254,8 @@ cq_chol_kernel(const CqPanel* __restrict__ panels, const float* __restrict__ par
   for (int kb = 0; kb < kBlks; ++kb) {
     const int k0 = kb * kNb;
     if (warp == 0) {
-      // Phase 1: the diagonal block, row k0 + lane in lane < 16, and its inverse, a column per lane
-      float a[kNb], inv[kNb];
+      // Phase 1: the diagonal block's factor, row k0 + lane
+      float a[kNb];
       const int row = lane & (kNb - 1);
 #pragma unroll
       for (int j = 0; j < kNb; ++j) a[j] = A[(k0 + row) * kLd + k0 + j];
@@ -245,9 +264,12 @@ cq_chol_kernel(const CqPanel* __restrict__ panels, const float* __restrict__ par
       for (int j = 0; j < kNb; ++j) {
         const float d = __shfl_sync(0xffffffffu, a[j], j);
         neg = neg || !(d > 0.f);
-        const float l = sqrtf(d > 0.f ? d : 1.f);
-        inv[j] = 1.f / l;
-        a[j] = row == j ? l : a[j] * inv[j];
+        const float l = sqrtf(d > 0.f ? d : 1.f), inv = 1.f / l;
+        if (lane == j) {
+          diag[j] = l;
+          dinv[j] = inv;
+        }
+        a[j] = row == j ? l : a[j] * inv;
 #pragma unroll
         for (int k = 0; k < kNb; ++k) {
           if (k <= j) continue;
@@ -255,51 +277,36 @@ cq_chol_kernel(const CqPanel* __restrict__ panels, const float* __restrict__ par
           if (row >= k) a[k] = fmaf(-a[j], lk, a[k]);
         }
       }
-      // L Y = I: lane c solves column c; L's rows come from their lanes
-      float y[kNb];
+      if (lane < kNb)
 #pragma unroll
-      for (int i = 0; i < kNb; ++i) {
-        float s = row == i ? 1.f : 0.f;
-#pragma unroll
-        for (int k = 0; k < kNb; ++k)
-          if (k < i) s = fmaf(-__shfl_sync(0xffffffffu, a[k], i), y[k], s);
-        y[i] = i >= row ? s * inv[i] : 0.f;
-      }
-      if (lane < kNb) {
-#pragma unroll
-        for (int j = 0; j < kNb; ++j) A[(k0 + row) * kLd + k0 + j] = y[j];
-      }
+        for (int j = 0; j < kNb; ++j) LT[j][row] = a[j];
       if (neg && lane == 0) bad = 1;
     }
     __syncthreads();
-    // Phase 2.  With D = L_11^-1 (its transpose is in A), rows below: L_21 = G_21 D^T (4 of a
-    // row's 16 entries an item); columns to the left: L^-1's rows k0 .. are -D times what phase
-    // 3 has summed there (4 rows of a column an item).  In place, so computed before written.
+    // Phase 2, a thread each: a row below, L_21 (its 16 entries by substitution from the left);
+    // or a column of L^-1's rows k0 .. (from what phase 3 has summed there, or the unit column).
     const int n_rows = R - k0 - kNb;
-    float v[4] = {0.f, 0.f, 0.f, 0.f};
-    float* o = nullptr;
-    if (tid < 4 * n_rows) {
-      const float* x = A + (k0 + kNb + tid / 4) * kLd + k0;
-      const float* y = A + k0 * kLd + k0 + 4 * (tid % 4);
+    if (tid < R) {
+      const bool below = tid < n_rows;
+      const int col = tid - n_rows;                        // of L^-1, < k0 + kNb
+      float* p = A + (below ? k0 + kNb + tid : col) * kLd + k0;
+      const int top = below ? -1 : col - k0;               // >= 0: the column's pivot row
+      float x[kNb];
 #pragma unroll
-      for (int k = 0; k < kNb; ++k)
+      for (int j = 0; j < kNb; ++j) x[j] = top >= 0 ? 0.f : p[j];
 #pragma unroll
-        for (int c = 0; c < 4; ++c) v[c] = fmaf(x[k], y[k * kLd + c], v[c]);
-      o = A + (k0 + kNb + tid / 4) * kLd + k0 + 4 * (tid % 4);
-    } else if (tid < 4 * (n_rows + k0)) {
-      const int rq = (tid - 4 * n_rows) / k0, col = (tid - 4 * n_rows) % k0;
-      const float* x = A + k0 * kLd + k0 + 4 * rq;
-      const float* y = A + col * kLd + k0;
+      for (int j = 0; j < kNb; ++j) {
+        if (below) x[j] *= dinv[j];
+        else if (j > top) x[j] = -x[j] / diag[j];
+        else if (j == top) x[j] = dinv[j];
+        const float m = below ? -x[j] : x[j];
 #pragma unroll
-      for (int k = 0; k < kNb; ++k)
+        for (int k = 0; k < kNb; ++k)
+          if (k > j) x[k] = fmaf(m, LT[j][k], x[k]);
+      }
 #pragma unroll
-        for (int c = 0; c < 4; ++c) v[c] = fmaf(-x[k * kLd + c], y[k], v[c]);
-      o = A + col * kLd + k0 + 4 * rq;
+      for (int j = 0; j < kNb; ++j) p[j] = x[j];
     }
-    __syncthreads();
-    if (o != nullptr)
-#pragma unroll
-      for (int c = 0; c < 4; ++c) o[c] = v[c];
     __syncthreads();
     // Phase 3, in 4 x 4 tiles of rows nt apart (and columns nt or ct apart): G_22 -= L_21
     // L_21^T, lower triangle; and below row block k0 of L^-1, L_21 times it.
@@ -314,19 +321,20 @@ cq_chol_kernel(const CqPanel* __restrict__ panels, const float* __restrict__ par
 #pragma unroll
         for (int i = 0; i < 4; ++i)
 #pragma unroll
-          for (int j = 0; j < 4; ++j) s[i][j] = 0.f;
+          for (int j = 0; j < 4; ++j)
+            if (j < i || (j == i && tj <= ti)) s[i][j] = g[i * nt * kLd + j * nt];
 #pragma unroll
         for (int k = 0; k < kNb; ++k)
 #pragma unroll
           for (int i = 0; i < 4; ++i)
 #pragma unroll
             for (int j = 0; j < 4; ++j)
-              if (j <= i) s[i][j] = fmaf(x[i * nt * kLd + k], y[j * nt * kLd + k], s[i][j]);
+              if (j <= i) s[i][j] = fmaf(-x[i * nt * kLd + k], y[j * nt * kLd + k], s[i][j]);
 #pragma unroll
         for (int i = 0; i < 4; ++i)
 #pragma unroll
           for (int j = 0; j < 4; ++j)
-            if (j < i || (j == i && tj <= ti)) g[i * nt * kLd + j * nt] -= s[i][j];
+            if (j < i || (j == i && tj <= ti)) g[i * nt * kLd + j * nt] = s[i][j];
       } else {
         float s[4][4];
         const int ti = (w - nt * nt) / ct, tj = (w - nt * nt) % ct;
@@ -453,25 +461,25 @@ cudaError_t run_cholqr_r(const CqPanel* d_panels, int32_t n_panels, const CqChun
   cudaError_t e = cudaFuncSetAttribute(cq_chol_kernel<R>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)chol_smem<R>());
   if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(cq_gram_kernel<R, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)Gram<R, true>::kSmem);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(cq_gram_kernel<R, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)Gram<R, false>::kSmem);
-  if (e == cudaSuccess)
     e = cudaFuncSetAttribute(cq_apply_kernel<R>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)Apply<R>::kSmem);
   if (e != cudaSuccess) return e;
+  constexpr int kT = R == 16 ? 2 : R == 32 ? 4 : 8, kG = R == 64 ? 8 : R == 128 ? 1 : 4;
+  constexpr int kSmallT = R == 16 ? 2 : R == 128 ? 8 : 4;
+  // fewer than four chunks per SM: a CTA each (r = 64: 4 x 4 tiles).  One 4096 x 4096 matrix
+  // 432 -> 189 us at r = 64, 109 -> 70 at r = 16.
+  const bool few = n_chunks < 608;
   // CTAs per chunk of 256-row parts: one each, or two parts (L^-1 read half as often)
-  const int n_split = R >= 64 || n_chunks < 608 ? cq_chunk_rows(R) / 256 : cq_chunk_rows(R) / 512;
+  const int n_split = kCqChunkRows / (R >= 64 || few ? 256 : 512);
   // first Cholesky QR: Omega -> Q1; second: Q1 -> Q; both in the panels
   for (int round = 0; round < 2; ++round) {
-    if (round == 0)
-      cq_gram_kernel<R, true><<<n_chunks, Gram<R, true>::kThreads, Gram<R, true>::kSmem, s>>>(
-          d_panels, d_chunks, d_partial, seed, refresh_idx);
+    if (few)
+      e = round == 0 ? launch_gram<R, kSmallT, 1, true>(d_panels, d_chunks, n_chunks, d_partial, seed, refresh_idx, s)
+                     : launch_gram<R, kSmallT, 1, false>(d_panels, d_chunks, n_chunks, d_partial, seed, refresh_idx, s);
     else
-      cq_gram_kernel<R, false><<<n_chunks, Gram<R, false>::kThreads, Gram<R, false>::kSmem, s>>>(
-          d_panels, d_chunks, d_partial, seed, refresh_idx);
+      e = round == 0 ? launch_gram<R, kT, kG, true>(d_panels, d_chunks, n_chunks, d_partial, seed, refresh_idx, s)
+                     : launch_gram<R, kT, kG, false>(d_panels, d_chunks, n_chunks, d_partial, seed, refresh_idx, s);
+    if (e != cudaSuccess) return e;
     e = launch_dependent(cq_chol_kernel<R>, (unsigned)(n_panels * kCholCtas), kCholThreads<R>,
                          chol_smem<R>(), s, kCholCtas, false, d_panels, d_partial, d_linv, d_status);
     if (e != cudaSuccess) return e;

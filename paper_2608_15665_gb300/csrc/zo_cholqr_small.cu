@@ -1,4 +1,4 @@
-// Subspace refresh at r = 4 and 8: Alg. 1's Haar factor of every panel in one launch, the
+// Subspace refresh of fp32 weights at r = 4 and 8: Alg. 1's Haar factor of every panel in one launch, the
 // panel held in registers.
 //
 // Tall panels (rows >= 4 r, at most 8 CTAs' worth) by CholeskyQR2 as in zo_cholqr.cu -- the
@@ -45,7 +45,7 @@ __device__ __forceinline__ void draw_row(const CqPanel& pn, int64_t row, uint64_
                                          uint32_t refresh_idx, float (&x)[R]) {
 #pragma unroll
   for (int c4 = 0; c4 < R / 4; ++c4) {
-    const float4 z = normal4(seed, (uint32_t)(row * (R / 4) + c4), pn.gidx, refresh_idx,
+    const float4 z = normal4_packed(seed, (uint32_t)(row * (R / 4) + c4), pn.gidx, refresh_idx,
                              query_word(pn.tag, 0));
     x[4 * c4] = z.x; x[4 * c4 + 1] = z.y; x[4 * c4 + 2] = z.z; x[4 * c4 + 3] = z.w;
   }

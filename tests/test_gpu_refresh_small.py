@@ -23,8 +23,8 @@ def test_panels_in_registers_match_oracle(lib, gpu, r):
     from paper_2608_15665_gb300.schedule import SubZeroPlus
     seed, base = 90 + r, 3
     # only U and V matter: one row of W per panel pair is enough for a wide matrix's memory
-    weights = [make_weight(m, n, "bf16", k, gpu, ldw=(n + 7) // 8 * 8) if m * n < 1 << 22
-               else torch.zeros(m, (n + 7) // 8 * 8, dtype=torch.bfloat16, device=gpu)[:, :n]
+    weights = [make_weight(m, n, "f32", k, gpu, ldw=(n + 3) // 4 * 4) if m * n < 1 << 22
+               else torch.zeros(m, (n + 3) // 4 * 4, device=gpu)[:, :n]
                for k, (m, n) in enumerate(CASES[r])]
     z = SubZeroPlus(weights, r, 2, seed, matrix_index_base=base)
     for j in (1, 2):

@@ -13,10 +13,10 @@ from parity import UV_ABS
 pytestmark = pytest.mark.gpu
 
 SHAPES = {
-    16: [(64, 65), (383, 385), (1023, 1025), (2047, 2049)],
-    32: [(128, 129), (191, 193), (1023, 1025), (2047, 2049)],
-    64: [(256, 257), (511, 513), (1023, 1025)],
-    128: [(512, 513), (543, 545), (1023, 1025)],
+    16: [(64, 65), (127, 129), (1023, 1025), (2047, 2049)],
+    32: [(128, 129), (255, 257), (1023, 1025), (2047, 2049)],
+    64: [(256, 257), (1023, 1025), (2047, 2049)],
+    128: [(512, 513), (1023, 1025), (2047, 2049)],
 }
 
 
@@ -43,3 +43,22 @@ def test_tall_panels_match_oracle(lib, gpu, r):
     s1 = snapshot(one)
     assert np.array_equal(s1["U"][0], s["U"][1]) and np.array_equal(s1["V"][0], s["V"][1])
     one.close()
+
+
+@pytest.mark.parametrize("r", [16, 32, 64])
+def test_many_chunks_have_the_bits_of_few(lib, gpu, r):
+    """More than 608 chunks (several per CTA, the last CTA's incomplete, panels of one and of two
+    chunks): each panel has the bits it has in a context of its own."""
+    from paper_2608_15665_gb300.schedule import SubZeroPlus
+    n = [(4 * r + 1, 4 * r + 37)] * 306 + [(1040, 4 * r)]
+    weights = [torch.zeros(a, (b + 7) // 8 * 8, dtype=torch.bfloat16, device=gpu)[:, :b] for a, b in n]
+    z = SubZeroPlus(weights, r, 2, 8)
+    z.refresh(1)
+    z.sync()
+    for i in (0, 1, 7, 8, 150, 304, 305, 306):
+        one = SubZeroPlus(weights[i:i + 1], r, 2, 8, matrix_index_base=i)
+        one.refresh(1)
+        one.sync()
+        assert torch.equal(one.U[0], z.U[i]) and torch.equal(one.V[0], z.V[i]), i
+        one.close()
+    z.close()
