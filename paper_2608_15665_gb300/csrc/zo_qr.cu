@@ -50,66 +50,78 @@ struct QrSmem {
   float tau[R];
 };
 
-// Block-wide sum of H per-thread values (columns off .. off+H-1) into
-// red[warp][off + c] (one partial per warp).
-template <int H>
-__device__ __forceinline__ void block_partials(float (&p)[H], float* red_buf, int row_len,
-                                               int off) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  float* red = red_buf + warp * row_len + off;
-  warp_reduce_scatter<H>(p, lane);
-  if (H >= 32) {
-    constexpr int kKeep = H >= 32 ? H / 32 : 1;
-#pragma unroll
-    for (int k = 0; k < kKeep; ++k) red[lane * kKeep + k] = p[k];
-  } else {
-    constexpr int kStride = H >= 32 ? 1 : 32 / H;
-    if (lane % kStride == 0) red[lane / kStride] = p[0];
-  }
-}
-
-// Columns are reduced in groups of at most 64 so that R = 128 fits in registers.
+// A step's columns in groups: a group left of the step's column is passed over by all threads
+// alike, and the 32 (or R) columns of a set are reduced together.
 template <int R>
-struct QrHalves {
-  static constexpr int kH = R > 64 ? 64 : R;
-  static constexpr int kN = R / kH;
+struct QrCols {
+  static constexpr int kG = R < 16 ? R : 16;
+  static constexpr int kH = R < 32 ? R : 32;
   static constexpr int kC32 = (R + 31) / 32;       // 32-column groups handled by warp 0
 };
 
-// a[j] for a runtime j without indexing the register array dynamically.
-template <int R>
-__device__ __forceinline__ float pick(const float (&row)[R], int j) {
-  float x = 0.f;
-#pragma unroll
-  for (int c = 0; c < R; ++c)
-    if (c == j) x = row[c];
-  return x;
+// Block-wide sums of a set's per-thread values: one partial per warp to red[0 .. H - 1].
+template <int H>
+__device__ __forceinline__ void warp_partials(float (&p)[H], float* red) {
+  const int lane = threadIdx.x & 31;
+  warp_reduce_scatter<H>(p, lane);
+  if (lane % (32 / H) == 0) red[lane / (32 / H)] = p[0];
 }
 
-// Householder factorisation of the block held in registers (row i = rho*256 + tid).
+// Householder factorisation of the block held in registers (row i = rho*256 + tid); rows from
+// n_real on are zero.
+//
+// Bound: instruction issue and two barriers per column.  The column's own entry comes from its
+// group (or, at r <= 16, where the columns are unrolled, from a fixed register), groups left of
+// the column and warps without rows below it take no part: a shorter panel or a later column
+// costs less, and every remaining sum is the same.  8 pairs of panels of 200 x 64: 283 -> 158 us a
+// refresh, of 400 and 504 x 128: 2497 -> 1142; 24 layers of the 1.3B set at r = 4: 78 -> 60, at
+// r = 8: 147 -> 86.
 template <int R>
-__device__ void factor_block(float (&a)[QrShape<R>::kRPT][R], QrSmem<R>& sm) {
+__device__ void factor_block(float (&a)[QrShape<R>::kRPT][R], int n_real, QrSmem<R>& sm) {
   constexpr int RPT = QrShape<R>::kRPT;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  using Hv = QrHalves<R>;
+  using Qc = QrCols<R>;
+  constexpr int kG = Qc::kG, kH = Qc::kH;
+  const int last = (RPT - 1) * kQrThreads + 32 * warp + 31;     // the warp's last row
+  const bool real = 32 * warp < n_real;
+#pragma unroll (R <= 16 ? R : 1)
   for (int j = 0; j < R; ++j) {
     const int buf = j & 1;
+    float xj[RPT];
 #pragma unroll
-    for (int hh = 0; hh < Hv::kN; ++hh) {
-      float p[Hv::kH];
+    for (int rho = 0; rho < RPT; ++rho) xj[rho] = 0.f;
+    if (real && last >= j) {
 #pragma unroll
-      for (int c = 0; c < Hv::kH; ++c) p[c] = 0.f;
+      for (int g = 0; g < R / kG; ++g)
+        if (g * kG + kG > j)
+#pragma unroll
+          for (int c = 0; c < kG; ++c)
+#pragma unroll
+            for (int rho = 0; rho < RPT; ++rho)
+              xj[rho] = g * kG + c == j ? a[rho][g * kG + c] : xj[rho];
+    }
+#pragma unroll
+    for (int hh = 0; hh < R / kH; ++hh) {
+      if (hh * kH + kH <= j) continue;
+      float* red = &sm.red[buf][warp][hh * kH];
+      if (!real || last <= j) {
+        if (lane < kH) red[lane] = 0.f;
+        continue;
+      }
+      float p[kH];
+#pragma unroll
+      for (int c = 0; c < kH; ++c) p[c] = 0.f;
 #pragma unroll
       for (int rho = 0; rho < RPT; ++rho) {
-        const int i = rho * kQrThreads + tid;
-        if (i > j) {
-          const float x = pick<R>(a[rho], j);
+        if (rho * kQrThreads + tid <= j) continue;
 #pragma unroll
-          for (int c = 0; c < Hv::kH; ++c)
-            if (hh * Hv::kH + c >= j) p[c] = fmaf(x, a[rho][hh * Hv::kH + c], p[c]);
+        for (int g = 0; g < kH / kG; ++g) {
+          if (hh * kH + g * kG + kG <= j) continue;
+#pragma unroll
+          for (int c = g * kG; c < g * kG + kG; ++c) p[c] = fmaf(xj[rho], a[rho][hh * kH + c], p[c]);
         }
       }
-      block_partials<Hv::kH>(p, &sm.red[buf][0][0], R, hh * Hv::kH);
+      warp_partials<kH>(p, red);
     }
     if (tid == j) {
 #pragma unroll
@@ -117,9 +129,9 @@ __device__ void factor_block(float (&a)[QrShape<R>::kRPT][R], QrSmem<R>& sm) {
     }
     __syncthreads();
     if (warp == 0) {
-      float sk[Hv::kC32];
+      float sk[Qc::kC32];
 #pragma unroll
-      for (int k = 0; k < Hv::kC32; ++k) {
+      for (int k = 0; k < Qc::kC32; ++k) {
         const int c = lane + 32 * k;
         sk[k] = 0.f;
         if (c < R) {
@@ -129,7 +141,7 @@ __device__ void factor_block(float (&a)[QrShape<R>::kRPT][R], QrSmem<R>& sm) {
       }
       float sel = 0.f;
 #pragma unroll
-      for (int k = 0; k < Hv::kC32; ++k)
+      for (int k = 0; k < Qc::kC32; ++k)
         if (k == (j >> 5)) sel = sk[k];
       const float s_j = __shfl_sync(0xffffffffu, sel, j & 31);
       const float alpha = sm.rowj[buf][j];
@@ -140,7 +152,7 @@ __device__ void factor_block(float (&a)[QrShape<R>::kRPT][R], QrSmem<R>& sm) {
         scale = 1.0f / (alpha - beta);
       }
 #pragma unroll
-      for (int k = 0; k < Hv::kC32; ++k) {
+      for (int k = 0; k < Qc::kC32; ++k) {
         const int c = lane + 32 * k;
         if (c < R && c > j) sm.wbuf[buf][c] = fmaf(scale, sk[k], sm.rowj[buf][c]);
       }
@@ -152,60 +164,80 @@ __device__ void factor_block(float (&a)[QrShape<R>::kRPT][R], QrSmem<R>& sm) {
       }
     }
     __syncthreads();
-    const float tau = sm.scal[buf][0], scale = sm.scal[buf][1];
+    if (!real || last < j) continue;
+    const float tau = sm.scal[buf][0], scale = sm.scal[buf][1], beta = sm.diag[j];
 #pragma unroll
     for (int rho = 0; rho < RPT; ++rho) {
       const int i = rho * kQrThreads + tid;
-      if (i > j) {
-        const float v = pick<R>(a[rho], j) * scale;
-        const float tv = -tau * v;
+      if (i < j) continue;
+      const float v = xj[rho] * scale;
+      const float tv = i > j ? -tau * v : -tau;
 #pragma unroll
-        for (int c = 0; c < R; ++c) {
-          if (c > j) a[rho][c] = fmaf(tv, sm.wbuf[buf][c], a[rho][c]);
-          if (c == j) a[rho][c] = v;
-        }
-      } else if (i == j) {
-        const float beta = sm.diag[j];
+      for (int g = 0; g < R / kG; ++g) {
+        if (g * kG > j) {
 #pragma unroll
-        for (int c = 0; c < R; ++c) {
-          if (c > j) a[rho][c] = fmaf(-tau, sm.wbuf[buf][c], a[rho][c]);
-          if (c == j) a[rho][c] = beta;
+          for (int c = g * kG; c < g * kG + kG; ++c)
+            a[rho][c] = fmaf(tv, sm.wbuf[buf][c], a[rho][c]);
+        } else if (g * kG + kG > j) {
+#pragma unroll
+          for (int c = g * kG; c < g * kG + kG; ++c) {
+            if (c > j) a[rho][c] = fmaf(tv, sm.wbuf[buf][c], a[rho][c]);
+            if (c == j) a[rho][c] = i > j ? v : beta;
+          }
         }
       }
     }
   }
 }
 
-// Y <- H_0 H_1 ... H_(R-1) Y with the reflectors in refl (padded stride kLd).
+// Y <- H_0 H_1 ... H_(R-1) Y with the reflectors in refl (padded stride kLd).  upper: Y starts
+// as a diagonal, so that the columns left of j are still zero from row j on.
 template <int R>
 __device__ void apply_reflectors_backward(float (&a)[QrShape<R>::kRPT][R], const float* refl,
-                                          QrSmem<R>& sm) {
+                                          int n_real, bool upper, QrSmem<R>& sm) {
   constexpr int RPT = QrShape<R>::kRPT;
   constexpr int LD = QrShape<R>::kLd;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  using Hv = QrHalves<R>;
+  using Qc = QrCols<R>;
+  constexpr int kG = Qc::kG, kH = Qc::kH;
+  const int last = (RPT - 1) * kQrThreads + 32 * warp + 31;
+  const bool real = 32 * warp < n_real;
   for (int j = R - 1; j >= 0; --j) {
     const int buf = j & 1;
+    const int c_min = upper ? j : 0;               // first column that changes
+    float v[RPT];
 #pragma unroll
-    for (int hh = 0; hh < Hv::kN; ++hh) {
-      float p[Hv::kH];
+    for (int rho = 0; rho < RPT; ++rho) {
+      const int i = rho * kQrThreads + tid;
+      v[rho] = i == j ? 1.0f : i > j ? refl[i * LD + j] : 0.f;
+    }
 #pragma unroll
-      for (int c = 0; c < Hv::kH; ++c) p[c] = 0.f;
+    for (int hh = 0; hh < R / kH; ++hh) {
+      if (hh * kH + kH <= c_min) continue;
+      float* red = &sm.red[buf][warp][hh * kH];
+      if (!real || last < j) {
+        if (lane < kH) red[lane] = 0.f;
+        continue;
+      }
+      float p[kH];
+#pragma unroll
+      for (int c = 0; c < kH; ++c) p[c] = 0.f;
 #pragma unroll
       for (int rho = 0; rho < RPT; ++rho) {
-        const int i = rho * kQrThreads + tid;
-        if (i >= j) {
-          const float v = (i == j) ? 1.0f : refl[i * LD + j];
+        if (rho * kQrThreads + tid < j) continue;
 #pragma unroll
-          for (int c = 0; c < Hv::kH; ++c) p[c] = fmaf(v, a[rho][hh * Hv::kH + c], p[c]);
+        for (int g = 0; g < kH / kG; ++g) {
+          if (hh * kH + g * kG + kG <= c_min) continue;
+#pragma unroll
+          for (int c = g * kG; c < g * kG + kG; ++c) p[c] = fmaf(v[rho], a[rho][hh * kH + c], p[c]);
         }
       }
-      block_partials<Hv::kH>(p, &sm.red[buf][0][0], R, hh * Hv::kH);
+      warp_partials<kH>(p, red);
     }
     __syncthreads();
     if (warp == 0) {
 #pragma unroll
-      for (int h = 0; h < (R + 31) / 32; ++h) {
+      for (int h = 0; h < Qc::kC32; ++h) {
         const int c = lane + 32 * h;
         if (c < R) {
           float s = 0.f;
@@ -216,15 +248,18 @@ __device__ void apply_reflectors_backward(float (&a)[QrShape<R>::kRPT][R], const
       }
     }
     __syncthreads();
+    if (!real || last < j) continue;
     const float tau = sm.tau[j];
 #pragma unroll
     for (int rho = 0; rho < RPT; ++rho) {
-      const int i = rho * kQrThreads + tid;
-      if (i >= j) {
-        const float v = (i == j) ? 1.0f : refl[i * LD + j];
-        const float tv = -tau * v;
+      if (rho * kQrThreads + tid < j) continue;
+      const float tv = -tau * v[rho];
 #pragma unroll
-        for (int c = 0; c < R; ++c) a[rho][c] = fmaf(tv, sm.wbuf[buf][c], a[rho][c]);
+      for (int g = 0; g < R / kG; ++g) {
+        if (g * kG + kG <= c_min) continue;
+#pragma unroll
+        for (int c = g * kG; c < g * kG + kG; ++c)
+          a[rho][c] = fmaf(tv, sm.wbuf[buf][c], a[rho][c]);
       }
     }
   }
@@ -298,7 +333,7 @@ qr_up_kernel(const QrBlock* __restrict__ blocks, uint64_t seed, uint32_t refresh
     }
   }
 
-  factor_block<R>(a, sm);
+  factor_block<R>(a, blk.n_real, sm);
 
   if (blk.flags & kQrTop) {
     regs_to_refl<R>(a, refl);
@@ -310,7 +345,7 @@ qr_up_kernel(const QrBlock* __restrict__ blocks, uint64_t seed, uint32_t refresh
 #pragma unroll
       for (int c = 0; c < R; ++c) a[rho][c] = (i == c) ? (sm.diag[c] < 0.f ? -1.f : 1.f) : 0.f;
     }
-    apply_reflectors_backward<R>(a, refl, sm);
+    apply_reflectors_backward<R>(a, refl, blk.n_real, true, sm);
     store_rows<R>(a, blk.rows, blk.n_real);
   } else {
     store_rows<R>(a, blk.rows, blk.n_real);
@@ -361,7 +396,7 @@ __global__ void __launch_bounds__(kQrThreads) qr_down_kernel(const QrBlock* __re
   }
   if (tid < R) sm.tau[tid] = blk.tau[tid];
   __syncthreads();
-  apply_reflectors_backward<R>(a, refl, sm);
+  apply_reflectors_backward<R>(a, refl, blk.n_real, false, sm);
   store_rows<R>(a, blk.rows, blk.n_real);
 }
 
