@@ -29,9 +29,9 @@
 // in packed multiply-adds, which shared memory can feed; only the Gram matrix's lower blocks;
 // only L^-1's lower half where a thread's columns allow; Omega drawn once; and a blocked
 // Cholesky.
-// Refresh of 16 layers of the 32B set at r = 64: 2.64 -> 1.91 ms; of 32 of the 7B set at r = 32:
-// 1.29 -> 0.93, of one 0.191 -> 0.141; of 8 at r = 128: 4.38 -> 1.88; of 24 of the 1.3B set at
-// r = 16: 0.278 -> 0.204.
+// Refresh of 16 layers of the 32B set at r = 64: 2.64 -> 1.70 ms; of 32 of the 7B set at r = 32:
+// 1.29 -> 0.90, of one 0.191 -> 0.141; of 8 at r = 128: 4.38 -> 1.82; of 24 of the 1.3B set at
+// r = 16: 0.278 -> 0.186.
 #include "zo_cluster.cuh"
 #include "zo_fma_common.cuh"
 #include "zo_kernels.h"
@@ -45,14 +45,15 @@ using namespace fma;
 // ---------------------------------------------------------------- Gram matrices of chunks
 // A CTA takes kG chunks; of each, T x T blocks of the lower triangle, a block per thread.  Every
 // element is one chain of fp32 multiply-adds over the chunk's rows in order, whatever the tile,
-// so the tile may follow the set: 8 x 8 at r = 64 and 128, where shared memory must feed the
-// multiply-adds; smaller ones, and one chunk per CTA, where chains are what is short.  256
-// threads load or draw a stage even where fewer multiply (one 7B layer at r = 32, CTAs of the
-// 64 that multiply: 205 us a refresh; of 256: 141).  Rows pass through a ring of stages, copied
-// two ahead or drawn one ahead.
+// so tiles are free to follow the machine: 4 x 4 (2 x 2 at r = 16), because chains are what is
+// short.  8 x 8 tiles load half as much from shared memory per multiply-add but leave a quarter
+// of the warps: 1.91 ms for 16 layers of the 32B set at r = 64 where these take 1.70, 1.17
+// against 0.89 for 32 of the 7B set at r = 32.  256 threads load or draw a stage even where fewer
+// multiply (one 7B layer at r = 32, CTAs of the 64 that multiply: 205 us a refresh; of 256: 141).
+// Rows pass through a ring of stages, copied two ahead or drawn one ahead.
 //
-// 4 layers of the 32B set at r = 64: 93 us (4 x 4 tiles, 512 chunks), where the bytes take 20 and
-// an 8 x 8 tile's multiply-adds and its shared-memory reads 34 each; Omega's draws add 63.
+// 4 layers of the 32B set at r = 64: 93 us, where the bytes take 20, the multiply-adds 34 and the
+// shared-memory reads 69; Omega's draws add 63.
 template <int R, int T, int kG, bool kOmega>
 struct Gram {
   static constexpr int kN = R / T;
@@ -60,7 +61,7 @@ struct Gram {
   static constexpr int kBlockThreads = (kBlocks * kG + 31) / 32 * 32;
   static constexpr int kThreads = kBlockThreads > 256 ? kBlockThreads : 256;
   static constexpr int kPer = 256 / kG;                               // loading threads of a chunk
-  static constexpr int kSub = kG > 4 ? 16 : kG > 1 ? 32 : R == 16 ? 128 : R == 32 ? 64 : 32;
+  static constexpr int kSub = kG > 1 ? 32 : R == 16 ? 128 : R == 32 ? 64 : 32;
   static constexpr int kStages = kOmega ? 2 : 3;
   static constexpr int kLd = R + 4;
   static constexpr int kStage = kG * kSub * kLd;                      // floats
@@ -154,7 +155,7 @@ cq_gram_kernel(const CqPanel* __restrict__ panels, const CqChunk* __restrict__ c
     if (!mine) continue;
     const int n = min(kSub, rows[g] - t * kSub);
     const float* X = cq_smem + t % kStages * Cfg::kStage + g * kSub * kLd;
-#pragma unroll (T == 8 ? 2 : 4)
+#pragma unroll 4
     for (int k = 0; k < n; ++k) {
       float2 a2[kP], b2[kP];
       load_pairs<T>(X + k * kLd + T * bi, a2);
@@ -464,18 +465,17 @@ cudaError_t run_cholqr_r(const CqPanel* d_panels, int32_t n_panels, const CqChun
     e = cudaFuncSetAttribute(cq_apply_kernel<R>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)Apply<R>::kSmem);
   if (e != cudaSuccess) return e;
-  constexpr int kT = R == 16 ? 2 : R == 32 ? 4 : 8, kG = R == 64 ? 8 : R == 128 ? 1 : 4;
-  constexpr int kSmallT = R == 16 ? 2 : R == 128 ? 8 : 4;
-  // fewer than four chunks per SM: a CTA each (r = 64: 4 x 4 tiles).  One 4096 x 4096 matrix
-  // 432 -> 189 us at r = 64, 109 -> 70 at r = 16.
+  constexpr int kT = R == 16 ? 2 : 4, kG = R == 128 ? 1 : 2;
+  // fewer than four chunks per SM: a CTA each (two: one 4096 x 4096 matrix at r = 64
+  // 246 us a refresh instead of 190, one 7B layer at r = 32 160 instead of 141)
   const bool few = n_chunks < 608;
   // CTAs per chunk of 256-row parts: one each, or two parts (L^-1 read half as often)
   const int n_split = kCqChunkRows / (R >= 64 || few ? 256 : 512);
   // first Cholesky QR: Omega -> Q1; second: Q1 -> Q; both in the panels
   for (int round = 0; round < 2; ++round) {
     if (few)
-      e = round == 0 ? launch_gram<R, kSmallT, 1, true>(d_panels, d_chunks, n_chunks, d_partial, seed, refresh_idx, s)
-                     : launch_gram<R, kSmallT, 1, false>(d_panels, d_chunks, n_chunks, d_partial, seed, refresh_idx, s);
+      e = round == 0 ? launch_gram<R, kT, 1, true>(d_panels, d_chunks, n_chunks, d_partial, seed, refresh_idx, s)
+                     : launch_gram<R, kT, 1, false>(d_panels, d_chunks, n_chunks, d_partial, seed, refresh_idx, s);
     else
       e = round == 0 ? launch_gram<R, kT, kG, true>(d_panels, d_chunks, n_chunks, d_partial, seed, refresh_idx, s)
                      : launch_gram<R, kT, kG, false>(d_panels, d_chunks, n_chunks, d_partial, seed, refresh_idx, s);
