@@ -29,9 +29,9 @@
 // in packed multiply-adds, which shared memory can feed; only the Gram matrix's lower blocks;
 // only L^-1's lower half where a thread's columns allow; Omega drawn once; and a blocked
 // Cholesky.
-// Refresh of 16 layers of the 32B set at r = 64: 2.64 -> 1.70 ms; of 32 of the 7B set at r = 32:
-// 1.29 -> 0.90, of one 0.191 -> 0.141; of 8 at r = 128: 4.38 -> 1.82; of 24 of the 1.3B set at
-// r = 16: 0.278 -> 0.186.
+// Refresh of 16 layers of the 32B set at r = 64: 2.64 -> 1.62 ms; of 32 of the 7B set at r = 32:
+// 1.29 -> 0.88, of one 0.191 -> 0.141; of 8 at r = 128: 4.38 -> 1.82; of 24 of the 1.3B set at
+// r = 16: 0.278 -> 0.182.
 #include "zo_cluster.cuh"
 #include "zo_fma_common.cuh"
 #include "zo_kernels.h"
@@ -371,21 +371,23 @@ cq_chol_kernel(const CqPanel* __restrict__ panels, const float* __restrict__ par
 // out[j][a] = sum_{b <= a} X[j][b] Linv[a][b] over one chunk, in place, in tiles of kRows rows:
 // dealt to gridDim.y CTAs, X and Linv's transpose LT[b][a] row-major in shared memory.  Thread
 // (ry, tx) owns rows ry + kRowThreads i and columns 4 tx .. + 3 of either half of the columns;
-// past half of b only the second half's are left.  4 layers of the 32B set at r = 64: 79 us
-// (31 for the bytes, 44 for the multiply-adds, 49 for the shared-memory reads).
-constexpr int kApplyThreads = 256;
+// past half of b only the second half's are left.  Several small CTAs per SM overlap one's copies
+// with the others' multiply-adds (two of 256 threads on 256 rows: a refresh of 16 layers of the
+// 32B set at r = 64 1.70 ms; four of 128 on 128 rows: 1.62).  Of about 70 us for 4 layers, 31
+// are for the bytes, 44 for the multiply-adds and 49 for the shared-memory reads.
 template <int R>
 struct Apply {
+  static constexpr int kThreads = R == 128 ? 256 : 128;
   static constexpr int kColThreads = R / 8;
-  static constexpr int kRowThreads = kApplyThreads / kColThreads;     // 128, 64, 32, 16
+  static constexpr int kRowThreads = kThreads / kColThreads;          // 64, 32, 16, 16
   static constexpr int kTR = R == 16 ? 2 : R == 64 ? 8 : 4;           // rows per thread
-  static constexpr int kRows = kRowThreads * kTR;                     // 256; 64 at R = 128
+  static constexpr int kRows = kRowThreads * kTR;                     // 128; 64 at R = 128
   static constexpr int kLd = R + 4;
   static constexpr size_t kSmem = sizeof(float) * ((size_t)kRows + R) * kLd;
 };
 
 template <int R>
-__global__ void __launch_bounds__(kApplyThreads, R <= 32 ? 3 : 2)
+__global__ void __launch_bounds__(Apply<R>::kThreads, R <= 32 ? 6 : R == 64 ? 4 : 2)
 cq_apply_kernel(const CqPanel* __restrict__ panels, const CqChunk* __restrict__ chunks,
                 const float* __restrict__ linv) {
   using Cfg = Apply<R>;
@@ -397,13 +399,13 @@ cq_apply_kernel(const CqPanel* __restrict__ panels, const CqChunk* __restrict__ 
   const CqPanel pn = panels[ch.panel];
   const int tid = threadIdx.x, tx = tid % Cfg::kColThreads, ry = tid / Cfg::kColThreads;
   const float* L = linv + (int64_t)ch.panel * R * R;
-  for (int w = tid; w < R * kW; w += kApplyThreads)
+  for (int w = tid; w < R * kW; w += Cfg::kThreads)
     cp_async_16(LT + (w / kW) * kLd + 4 * (w % kW), L + 4 * w, 16);
   for (int s0 = blockIdx.y * Cfg::kRows; s0 < ch.nrows; s0 += gridDim.y * Cfg::kRows) {
     const int n = min(Cfg::kRows, ch.nrows - s0);
     float* rows = pn.out + (ch.row0 + s0) * R;
     __syncthreads();
-    for (int w = tid; w < n * kW; w += kApplyThreads)
+    for (int w = tid; w < n * kW; w += Cfg::kThreads)
       cp_async_16(X + (w / kW) * kLd + 4 * (w % kW), rows + 4 * (int64_t)w, 16);
     cp_async_commit();
     cp_async_wait<0>();
@@ -469,8 +471,9 @@ cudaError_t run_cholqr_r(const CqPanel* d_panels, int32_t n_panels, const CqChun
   // fewer than four chunks per SM: a CTA each (two: one 4096 x 4096 matrix at r = 64
   // 246 us a refresh instead of 190, one 7B layer at r = 32 160 instead of 141)
   const bool few = n_chunks < 608;
-  // CTAs per chunk of 256-row parts: one each, or two parts (L^-1 read half as often)
-  const int n_split = kCqChunkRows / (R >= 64 || few ? 256 : 512);
+  // CTAs per chunk: one tile each; at r = 128, two 64-row tiles of 16 where chunks are many, for
+  // L^-1's 64 KB (8 layers of the 7B set: 1.82 ms, one per CTA 1.84; one layer 476 and 467 us)
+  const int n_split = R < 128 || few ? 8 : 4;
   // first Cholesky QR: Omega -> Q1; second: Q1 -> Q; both in the panels
   for (int round = 0; round < 2; ++round) {
     if (few)
@@ -483,7 +486,7 @@ cudaError_t run_cholqr_r(const CqPanel* d_panels, int32_t n_panels, const CqChun
     e = launch_dependent(cq_chol_kernel<R>, (unsigned)(n_panels * kCholCtas), kCholThreads<R>,
                          chol_smem<R>(), s, kCholCtas, false, d_panels, d_partial, d_linv, d_status);
     if (e != cudaSuccess) return e;
-    cq_apply_kernel<R><<<dim3(n_chunks, n_split), kApplyThreads, Apply<R>::kSmem, s>>>(
+    cq_apply_kernel<R><<<dim3(n_chunks, n_split), Apply<R>::kThreads, Apply<R>::kSmem, s>>>(
         d_panels, d_chunks, d_linv);
   }
   return cudaGetLastError();
