@@ -112,8 +112,8 @@ enum {
                                      ~0.1 s and leave Y partly written.  Nothing faults; the
                                      context stays usable. */
   ZO_OPTION_LINEAR_TILE = 3, /* tiles (rows of X x columns of Y) of zo_linear_perturbed's
-                               Y = X W^T + S U^T GEMM: 0 = automatic (up to 128 tokens all of
-                               them x a few columns of Y per CTA, reported as tiling 9; else
+                               Y = X W^T + S U^T GEMM: 0 = automatic (up to 128 tokens at
+                               r <= 64 all of them x a few columns of Y per CTA, tiling 9; else
                                the SM-pair tiling whose busiest pair has the least operand
                                traffic; the single-CTA ones if no 2-CTA cluster fits),
                                1 = 128 x 256,

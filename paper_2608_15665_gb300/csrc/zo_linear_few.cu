@@ -1,5 +1,5 @@
 // The perturbed linear layer (Y = X W_i^T + S U_i^T, S = X P^T, the forward of Alg. 3 at
-// W' = W + eps U Z V^T, Eq. (4) form, with W left as it is) for at most 128 tokens, where
+// W' = W + eps U Z V^T, Eq. (4) form, with W left as it is) for at most 128 tokens at r <= 64, where
 // reading W_i is what there is to do.
 //
 // One CTA per SM owns all the tokens and `cols` columns of Y (rows of W_i; a multiple of 16
@@ -17,17 +17,18 @@
 // wait on nothing, so the waits cannot block the grid.
 //
 // K steps and the rank-r step's products are those of the SM-pair kernel, in its order, with
-// one accumulator per output: at r <= 64 Y has its bits (at r = 128 S is summed over one range
-// of K here).
+// one accumulator per output: Y has its bits.  (At r = 128 that kernel sums S over ranges of K
+// in fp32; one range here moved Y by up to rel 3.3e-5, so r = 128 stays with it, although
+// 4096 x 4096 took 18, 20 and 20 us at 1, 97 and 128 tokens here and takes 36, 53 and 60.)
 //
 // Bound: an output's chain of MMAs, about 85 cycles for each 16 elements of K however few the
 // columns (1024 x 12288: 38 us at any T), until the stream into the SM, 128 B per token and W
 // row for 64 elements of K, or HBM's 2 bytes per weight take longer (12288 x 12288: 49 us at
 // one token, 6.2 TB/s).  Measured at 1, 97 and 128 tokens, r = 32, against the SM-pair kernel's
 // best tiling: 4096 x 4096 17.6, 17.3, 17.3 us (28, 26, 26); 11008 x 4096 19.4, 20.2, 22.5 us
-// (41, 28, 29); 4096 x 11008 35, 37, 37 us (55, 54, 54); 4096 x 4096 at r = 128 18, 20, 20 us
-// (36, 53, 60).  Splitting K over a cluster of CTAs cuts the chain (4096 x 11008: 19 us at one
-// token) but sums in another order, and its exchange grows with the tokens (25 us at 97).
+// (41, 28, 29); 4096 x 11008 35, 37, 37 us (55, 54, 54).  Splitting K over a cluster of CTAs
+// cuts the chain (4096 x 11008: 19 us at one token) but sums in another order, and its exchange
+// grows with the tokens (25 us at 97).
 //
 // Roles (256 threads): warp 0 lane 0 loads by TMA, warp 1 lane 0 issues the MMAs (warp 1 owns
 // the Tensor Memory), then all eight warps empty the accumulator.  Every wait is bounded; a
@@ -93,7 +94,6 @@ linear_few_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
                   const __grid_constant__ CUtensorMap tm_s, const __grid_constant__ CUtensorMap tm_u,
                   const FewArgs a) {
   constexpr int kSC = s_cols(R);
-  constexpr int kExt = R == 128 ? 3 : 1;              // stages of the rank-r step
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
                                              ~uintptr_t(1023));
@@ -110,7 +110,7 @@ linear_few_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
   const int s_blk = is_s ? (int)blockIdx.x % (R / kSC) : 0;              // S: block of columns
   const int col0 = is_s ? 0 : ((int)blockIdx.x - a.n_s) * a.cols;
   const int k_stages = (a.k_steps + panels - 1) / panels;
-  const int n_k = is_s ? k_stages : k_stages + kExt;
+  const int n_k = is_s ? k_stages : k_stages + 1;         // and the rank-r step
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < S; ++s) {
@@ -169,23 +169,18 @@ linear_few_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
           }
         }
       } else {                               // the rank-r step: S_HL rows, U operand rows
-        const int j = k - k_stages;
-        if (j == 0) {
-          if (!wait_s_rows(a.flags, a.n_s, a.wait_epoch, abort, a.wait_cycles)) {
-            ok = false;
-            break;
-          }
-          fence_async_global();
+        if (!wait_s_rows(a.flags, a.n_s, a.wait_epoch, abort, a.wait_cycles)) {
+          ok = false;
+          break;
         }
-        // r <= 32: one panel [hi | lo | 0]; r = 64: the hi and the lo panel; r = 128: the hi
-        // panels, the hi ones of S and the lo ones of U, the lo ones of S and the hi ones of U
-        const int sx = j == 2 ? R : 0, ux = j == 1 ? R : 0;
+        fence_async_global();
+        // r <= 32: one panel [hi | lo | 0]; r = 64: the hi and the lo panel
         constexpr int kP = R <= 32 ? 1 : 2;
         mbar_arrive_expect_tx(&sh.full[s], (uint32_t)(kP * (a_panel + b_panel)));
 #pragma unroll
         for (int p = 0; p < kP; ++p) {
-          tma_load_2d(ap + p * a_panel, &tm_s, sx + 64 * p, 0, &sh.full[s]);
-          tma_load_2d(bp + p * b_panel, &tm_u, ux + 64 * p, a.u_row0 + col0, &sh.full[s]);
+          tma_load_2d(ap + p * a_panel, &tm_s, 64 * p, 0, &sh.full[s]);
+          tma_load_2d(bp + p * b_panel, &tm_u, 64 * p, a.u_row0 + col0, &sh.full[s]);
         }
       }
       ++n_st;
@@ -231,7 +226,7 @@ linear_few_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
           mma_f16(tmem, a0 + hi, b0 + lo, idesc, 1u);
           mma_f16(tmem, a0 + lo, b0 + hi, idesc, 1u);
         }
-      } else if constexpr (R == 64) {
+      } else {
 #pragma unroll
         for (int kk = 0; kk < 4; ++kk) {
           const uint64_t st = kk * kStepK;
@@ -239,12 +234,6 @@ linear_few_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
           mma_f16(tmem, a0 + st, b0 + pb + st, idesc, 1u);
           mma_f16(tmem, a0 + pa + st, b0 + st, idesc, 1u);
         }
-      } else {
-#pragma unroll
-        for (int p = 0; p < 2; ++p)
-#pragma unroll
-          for (int kk = 0; kk < 4; ++kk)
-            mma_f16(tmem, a0 + p * pa + kk * kStepK, b0 + p * pb + kk * kStepK, idesc, 1u);
       }
       mma_commit(&sh.empty[s]);
       if (++s == S) { s = 0; ph ^= 1u; }
@@ -337,7 +326,7 @@ int64_t ceil_div(int64_t a, int64_t b) { return (a + b - 1) / b; }
 
 LinearFewPlan linear_few_plan(int64_t T, int64_t m, int64_t n, int32_t r, int32_t sms) {
   LinearFewPlan pl{};
-  if (T < 1 || T > kMaxTokens || m < 1 || n < 1 || (r != 16 && r != 32 && r != 64 && r != 128))
+  if (T < 1 || T > kMaxTokens || m < 1 || n < 1 || (r != 16 && r != 32 && r != 64))
     return pl;
   pl.tokens = (int32_t)(ceil_div(T, 16) * 16);
   pl.s_cols = s_cols(r);
@@ -404,7 +393,6 @@ cudaError_t launch_linear_few(const CUtensorMap& tm_x, const CUtensorMap& tm_xs,
     ZO_FEW(16);
     ZO_FEW(32);
     ZO_FEW(64);
-    ZO_FEW(128);
     default: return cudaErrorInvalidValue;
   }
 #undef ZO_FEW

@@ -16,7 +16,7 @@ pytestmark = pytest.mark.gpu
 SHAPES = [(8 * 17, 136, 144), (128, 520, None), (136, 2056, None), (520, 4104, 4112), (264, 128, None)]
 
 
-@pytest.mark.parametrize("r", [16, 32, 64, 128])
+@pytest.mark.parametrize("r", [16, 32, 64])
 def test_few_tokens_match_oracle(lib, gpu, r):
     from paper_2608_15665_gb300 import binding as zb
     from paper_2608_15665_gb300.schedule import SubZeroPlus
@@ -39,7 +39,7 @@ def test_few_tokens_match_oracle(lib, gpu, r):
             tiling = zb.zo_linear_tiling(z.ctx)
             z.sync()
             took += tiling == 9
-            if tiling == 9 and r <= 64:
+            if tiling == 9:
                 # the SM-pair kernel's K steps and products, in its order: its bits
                 Yp = torch.empty(T, m, dtype=torch.bfloat16, device=gpu)
                 zb.zo_set_option(z.ctx, zb.ZO_OPTION_LINEAR_TILE, 8)
