@@ -40,13 +40,16 @@ __device__ __forceinline__ float ld_cluster(const float* p, uint32_t rank) {
   return v;
 }
 
-template <int R>
+// A row of Omega: the packed transform for tall panels; CUDA's functions for short ones, whose
+// condition number can turn a last place into 1e-5 of Q.
+template <int R, bool kTall>
 __device__ __forceinline__ void draw_row(const CqPanel& pn, int64_t row, uint64_t seed,
                                          uint32_t refresh_idx, float (&x)[R]) {
 #pragma unroll
   for (int c4 = 0; c4 < R / 4; ++c4) {
-    const float4 z = normal4_packed(seed, (uint32_t)(row * (R / 4) + c4), pn.gidx, refresh_idx,
-                             query_word(pn.tag, 0));
+    const uint32_t c = (uint32_t)(row * (R / 4) + c4);
+    const float4 z = kTall ? normal4_packed(seed, c, pn.gidx, refresh_idx, query_word(pn.tag, 0))
+                           : normal4(seed, c, pn.gidx, refresh_idx, query_word(pn.tag, 0));
     x[4 * c4] = z.x; x[4 * c4 + 1] = z.y; x[4 * c4 + 2] = z.z; x[4 * c4 + 3] = z.w;
   }
 }
@@ -58,8 +61,8 @@ __device__ __forceinline__ void store_row(const CqPanel& pn, int64_t row, const 
     out[c4] = make_float4(x[4 * c4], x[4 * c4 + 1], x[4 * c4 + 2], x[4 * c4 + 3]);
 }
 
-// One panel of at most 32 rows by one warp: Householder with row i in lane i (the convention
-// of zo_qr.cu), then Q = H_0 ... H_(R-1) [diag(sgn R_cc); 0], sgn(0) = +1.
+// One panel of at most 32 rows by one warp: Householder with row i in lane i (the convention,
+// sums and bits of zo_qr.cu), then Q = H_0 ... H_(R-1) [diag(sgn R_cc); 0], sgn(0) = +1.
 template <int R>
 __device__ __forceinline__ void short_panel(const CqPanel& pn, uint64_t seed, uint32_t refresh_idx) {
   const int lane = threadIdx.x & 31;
@@ -67,7 +70,7 @@ __device__ __forceinline__ void short_panel(const CqPanel& pn, uint64_t seed, ui
   float a[R];
 #pragma unroll
   for (int c = 0; c < R; ++c) a[c] = 0.f;
-  if (live) draw_row<R>(pn, lane, seed, refresh_idx, a);
+  if (live) draw_row<R, false>(pn, lane, seed, refresh_idx, a);
   float tau[R], diag[R];
 #pragma unroll
   for (int j = 0; j < R; ++j) {
@@ -137,7 +140,7 @@ cq_small_kernel(const CqPanel* __restrict__ tall, int n_tall, const CqPanel* __r
     const int64_t row = (int64_t)(k * ctas + rank) * kThreads + tid;
 #pragma unroll
     for (int c = 0; c < R; ++c) x[k][c] = 0.f;
-    if (row < pn.rows) draw_row<R>(pn, row, seed, refresh_idx, x[k]);
+    if (row < pn.rows) draw_row<R, true>(pn, row, seed, refresh_idx, x[k]);
   }
   bool bad = false;
 #pragma unroll 1

@@ -45,3 +45,21 @@ def test_panels_in_registers_match_oracle(lib, gpu, r):
     z.sync()
     assert all(torch.equal(x, y) for x, y in zip(a, z.U + z.V))
     z.close()
+
+
+@pytest.mark.parametrize("r", [4, 8])
+def test_short_panels_have_the_householder_panels_bits(lib, gpu, r):
+    """fp32 and bf16 weights of one index: panels shorter than 4r, whose condition number can be
+    large, are the same whichever kernel forms them."""
+    from paper_2608_15665_gb300.schedule import SubZeroPlus
+    shapes = [(r, r + 1), (2 * r - 1, 2 * r), (2 * r + 1, 4 * r - 1)]
+    sets = [[torch.zeros(m, (n + 7) // 8 * 8, dtype=dt, device=gpu)[:, :n] for m, n in shapes]
+            for dt in (torch.float32, torch.bfloat16)]
+    got = []
+    for weights in sets:
+        z = SubZeroPlus(weights, r, 2, 17, matrix_index_base=4)
+        z.refresh(2)
+        z.sync()
+        got.append([t.clone() for t in z.U + z.V])
+        z.close()
+    assert all(torch.equal(a, b) for a, b in zip(*got))
