@@ -43,17 +43,17 @@ L2_BYTES = 129e6          # GB300 L2 capacity
 TRAFFIC_BY_SOURCE = {
     # code hash of the kernel that runs (comments ignored) -> dram read + write bytes of one
     # launch, from an ncu capture on a small case of the same workload, scaled by weights
-    # profiles/wpass_tc_r32_llama7b_2layers.md: 1.5779 GB on the 2-layer subset, x16.0
-    ("a733f29ccdac1cbd", "llama7b_bf16_r32"): 25.25e9,
-    # profiles/wpass_pair_r128_llama7b_2layers.md: 1.6392 GB on the 2-layer subset, x16.0
-    ("45f2d025ab358fe7", "llama7b_bf16_r128_q99"): 26.23e9,
-    # profiles/wpass_tmem_r64_dense32b_1layer.md: 1.9271 GB on the 1-layer subset, x64.0
-    ("5d6c6cd8669a0a74", "dense32b_bf16_r64"): 123.33e9,
+    # profiles/wpass_tc_r32_llama7b_2layers.md: 1.5776 GB on the 2-layer subset, x16.0
+    ("32b0dddb3786330a", "llama7b_bf16_r32"): 25.24e9,
+    # profiles/wpass_pair_r128_llama7b_2layers.md: 1.6395 GB on the 2-layer subset, x16.0
+    ("d1d9e6f8246f6b1f", "llama7b_bf16_r128_q99"): 26.23e9,
+    # profiles/wpass_tmem_r64_dense32b_1layer.md: 1.9265 GB on the 1-layer subset, x64.0
+    ("2e37b0bf937bfe68", "dense32b_bf16_r64"): 123.30e9,
 }
 # thread instructions per weight of the full-space SPSA kernel (ncu), keyed by source hash
 INSTR_PER_WEIGHT_BY_SOURCE = {
-    # profiles/mezo_kernel_llama7b_2layers.md: 751.9 M warp instructions x 32 / 404.75 M weights
-    "a1a0ede2c35a3971": 59.4,
+    # profiles/mezo_kernel_llama7b_2layers.md: 482.6 M warp instructions x 32 / 404.75 M weights
+    "59503d8e1c27879d": 38.2,
 }
 
 
