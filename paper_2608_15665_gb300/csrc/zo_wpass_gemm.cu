@@ -17,7 +17,11 @@
 //    Three CTAs per SM overlap one's loads and stores with the others' arithmetic: at
 //    r = 32 and 64 that makes 64-row tiles faster than 128-row ones with two CTAs (164 and
 //    267 us against 176 and 295), elsewhere they are within 3%; 32-row tiles are slower
-//    (217 and 385 us).
+//    (217 and 385 us).  At r <= 16, where there is little arithmetic to hide W's latency under,
+//    four CTAs, at 64 registers: 121 -> 115 us at r = 16, 112 -> 105 at r = 8 (bf16: 85 -> 77);
+//    five or six spill (160 and 245 us at r = 8).  From r = 32 on, fewer, 8 x 8 register tiles
+//    read less from shared memory, of which the 4 x 8 ones take 67%, but leave too few warps
+//    (128 threads: 192 us at r = 32).
 #include "zo_fma_common.cuh"
 #include "zo_launch.cuh"
 
@@ -184,7 +188,7 @@ __device__ __forceinline__ void gemm_tile(const MatDesc& md, int64_t local, floa
 }
 
 template <int R>
-__global__ void __launch_bounds__(kGemmThreads, 3)
+__global__ void __launch_bounds__(kGemmThreads, R <= 16 ? 4 : 3)
 wpass_gemm_kernel(const MatDesc* __restrict__ mats, int n_mats, const int64_t* __restrict__ prefix) {
   extern __shared__ float4 smem4[];
   float* smem = reinterpret_cast<float*>(smem4);
