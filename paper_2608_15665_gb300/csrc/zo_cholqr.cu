@@ -30,7 +30,7 @@
 // only L^-1's lower half where a thread's columns allow; Omega drawn once; and a blocked
 // Cholesky.
 // Refresh of 16 layers of the 32B set at r = 64: 2.64 -> 1.62 ms; of 32 of the 7B set at r = 32:
-// 1.29 -> 0.88, of one 0.191 -> 0.141; of 8 at r = 128: 4.38 -> 1.82; of 24 of the 1.3B set at
+// 1.29 -> 0.88, of one 0.191 -> 0.132; of 8 at r = 128: 4.38 -> 1.82; of 24 of the 1.3B set at
 // r = 16: 0.278 -> 0.182.
 #include "zo_cluster.cuh"
 #include "zo_fma_common.cuh"
@@ -108,6 +108,10 @@ cq_gram_kernel(const CqPanel* __restrict__ panels, const CqChunk* __restrict__ c
     tag = query_word(pn.tag, 0);
   }
   if (w0 == 0 && tid < 256) rows[q] = words / kW;
+  if constexpr (kG == 1) {                       // the launches of few chunks are dependent
+    pdl_wait();
+    pdl_trigger();
+  }
   __syncthreads();
   const int g = min(tid / Cfg::kBlocks, kG - 1), u = tid % Cfg::kBlocks;
   int bi = 0;
@@ -185,14 +189,15 @@ cq_gram_kernel(const CqPanel* __restrict__ panels, const CqChunk* __restrict__ c
 
 template <int R, int T, int kG, bool kOmega>
 cudaError_t launch_gram(const CqPanel* d_panels, const CqChunk* d_chunks, int32_t n_chunks,
-                        float* d_partial, uint64_t seed, uint32_t refresh_idx, cudaStream_t s) {
+                        float* d_partial, uint64_t seed, uint32_t refresh_idx, bool dependent,
+                        cudaStream_t s) {
   using Cfg = Gram<R, T, kG, kOmega>;
   const cudaError_t e = cudaFuncSetAttribute(
       cq_gram_kernel<R, T, kG, kOmega>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg::kSmem);
   if (e != cudaSuccess) return e;
-  cq_gram_kernel<R, T, kG, kOmega><<<(n_chunks + kG - 1) / kG, Cfg::kThreads, Cfg::kSmem, s>>>(
-      d_panels, d_chunks, n_chunks, d_partial, seed, refresh_idx);
-  return cudaGetLastError();
+  return launch_dependent(cq_gram_kernel<R, T, kG, kOmega>, (unsigned)((n_chunks + kG - 1) / kG),
+                          Cfg::kThreads, Cfg::kSmem, s, 1, dependent, d_panels, d_chunks, n_chunks,
+                          d_partial, seed, refresh_idx);
 }
 
 // ---------------------------------------------------------------- Cholesky factor, inverse
@@ -232,6 +237,8 @@ cq_chol_kernel(const CqPanel* __restrict__ panels, const float* __restrict__ par
     if (tid == 0) bad = 0;
   }
   cta2::cluster_sync_all();                      // all CTAs of the cluster run
+  pdl_wait();
+  pdl_trigger();
   const uint32_t a0 = cta2::map_to(A, 0);
   for (int w = tid; w < R * R / 4 / kCholCtas; w += kThreads) {
     const int i = w / (R / 4) * kCholCtas + rank, j = 4 * (w % (R / 4));
@@ -399,6 +406,8 @@ cq_apply_kernel(const CqPanel* __restrict__ panels, const CqChunk* __restrict__ 
   const CqPanel pn = panels[ch.panel];
   const int tid = threadIdx.x, tx = tid % Cfg::kColThreads, ry = tid / Cfg::kColThreads;
   const float* L = linv + (int64_t)ch.panel * R * R;
+  pdl_wait();
+  pdl_trigger();
   for (int w = tid; w < R * kW; w += Cfg::kThreads)
     cp_async_16(LT + (w / kW) * kLd + 4 * (w % kW), L + 4 * w, 16);
   for (int s0 = blockIdx.y * Cfg::kRows; s0 < ch.nrows; s0 += gridDim.y * Cfg::kRows) {
@@ -468,28 +477,33 @@ cudaError_t run_cholqr_r(const CqPanel* d_panels, int32_t n_panels, const CqChun
                              (int)Apply<R>::kSmem);
   if (e != cudaSuccess) return e;
   constexpr int kT = R == 16 ? 2 : 4, kG = R == 128 ? 1 : 2;
-  // fewer than four chunks per SM: a CTA each (two: one 4096 x 4096 matrix at r = 64
-  // 246 us a refresh instead of 190, one 7B layer at r = 32 160 instead of 141)
+  // fewer than four chunks per SM: a CTA each (as ordinary launches; two per CTA: one 4096 x 4096
+  // matrix at r = 64 246 us a refresh instead of 190, one 7B layer at r = 32 160 instead of 141)
   const bool few = n_chunks < 608;
+  // Few chunks: launches that wait for their predecessor and overlap its tail (one 4096 x 4096
+  // matrix 185 -> 169 us at r = 64, 74 -> 59 at r = 16).  Not at r = 128, where the next kernel's
+  // large CTAs take the SM from this one's (one 7B layer: 467 -> 512 us).
+  const bool dep = few && R < 128;
   // CTAs per chunk: one tile each; at r = 128, two 64-row tiles of 16 where chunks are many, for
   // L^-1's 64 KB (8 layers of the 7B set: 1.82 ms, one per CTA 1.84; one layer 476 and 467 us)
   const int n_split = R < 128 || few ? 8 : 4;
   // first Cholesky QR: Omega -> Q1; second: Q1 -> Q; both in the panels
   for (int round = 0; round < 2; ++round) {
     if (few)
-      e = round == 0 ? launch_gram<R, kT, 1, true>(d_panels, d_chunks, n_chunks, d_partial, seed, refresh_idx, s)
-                     : launch_gram<R, kT, 1, false>(d_panels, d_chunks, n_chunks, d_partial, seed, refresh_idx, s);
+      e = round == 0 ? launch_gram<R, kT, 1, true>(d_panels, d_chunks, n_chunks, d_partial, seed, refresh_idx, dep, s)
+                     : launch_gram<R, kT, 1, false>(d_panels, d_chunks, n_chunks, d_partial, seed, refresh_idx, dep, s);
     else
-      e = round == 0 ? launch_gram<R, kT, kG, true>(d_panels, d_chunks, n_chunks, d_partial, seed, refresh_idx, s)
-                     : launch_gram<R, kT, kG, false>(d_panels, d_chunks, n_chunks, d_partial, seed, refresh_idx, s);
+      e = round == 0 ? launch_gram<R, kT, kG, true>(d_panels, d_chunks, n_chunks, d_partial, seed, refresh_idx, dep, s)
+                     : launch_gram<R, kT, kG, false>(d_panels, d_chunks, n_chunks, d_partial, seed, refresh_idx, dep, s);
     if (e != cudaSuccess) return e;
     e = launch_dependent(cq_chol_kernel<R>, (unsigned)(n_panels * kCholCtas), kCholThreads<R>,
-                         chol_smem<R>(), s, kCholCtas, false, d_panels, d_partial, d_linv, d_status);
+                         chol_smem<R>(), s, kCholCtas, dep, d_panels, d_partial, d_linv, d_status);
     if (e != cudaSuccess) return e;
-    cq_apply_kernel<R><<<dim3(n_chunks, n_split), Apply<R>::kThreads, Apply<R>::kSmem, s>>>(
-        d_panels, d_chunks, d_linv);
+    e = launch_dependent(cq_apply_kernel<R>, dim3(n_chunks, n_split), Apply<R>::kThreads,
+                         Apply<R>::kSmem, s, 1, dep, d_panels, d_chunks, d_linv);
+    if (e != cudaSuccess) return e;
   }
-  return cudaGetLastError();
+  return cudaSuccess;
 }
 
 }  // namespace

@@ -10,6 +10,9 @@
 // trigger: the next pass's coefficient kernel, resident beside them from their start, cost
 // the 7B set's r = 32 pass 4% (4.16 ms against 3.99).
 //
+// The refresh's launches are dependent ones where few chunks make them latency-bound
+// (zo_cholqr.cu).
+//
 // A pass of one 2048 x 2048 matrix at r = 32 went from 26.7 us (four ordinary launches) to
 // 16.2 us (three dependent ones).
 #pragma once
@@ -26,10 +29,10 @@ __device__ __forceinline__ void pdl_trigger() {
 // cluster: CTAs per cluster (1: none, or the kernel's own __cluster_dims__).  dependent =
 // false: an ordinary launch, after everything before it has completed.
 template <typename... Params, typename... Args>
-cudaError_t launch_dependent(void (*kernel)(Params...), unsigned grid, unsigned block, size_t smem,
+cudaError_t launch_dependent(void (*kernel)(Params...), dim3 grid, unsigned block, size_t smem,
                              cudaStream_t s, unsigned cluster, bool dependent, Args... args) {
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(grid, 1, 1);
+  cfg.gridDim = grid;
   cfg.blockDim = dim3(block, 1, 1);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
