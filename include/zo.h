@@ -171,7 +171,8 @@ ZO_API zo_status zo_destroy(zo_ctx* ctx);
  * and Omega_V (n x r, tag 3) from the counter contract and writes into U_i and V_i
  * the Q of their thin QR factorisation with diag(R) > 0, i.e. Q with column c
  * multiplied by sgn(R_cc) (Eq. (11), sgn(0) = +1).  That factor is unique; panels
- * with at least 4r rows at r >= 16 reach it by CholeskyQR2 (two rounds of Cholesky
+ * with at least 4r rows at r >= 16 (and tall ones of fp32 weights at r = 4 and 8)
+ * reach it by CholeskyQR2 (two rounds of Cholesky
  * of the Gram matrix and a triangular solve), the others by a batched Householder
  * TSQR with the sign fix.  A Gram matrix without a positive pivot (not expected for
  * such panels) makes the next zo_sync_status return ZO_ERR_CUDA.  reset_moments != 0
