@@ -408,6 +408,8 @@ cq_apply_kernel(const CqPanel* __restrict__ panels, const CqChunk* __restrict__ 
   const float* L = linv + (int64_t)ch.panel * R * R;
   pdl_wait();
   pdl_trigger();
+  // a short chunk leaves CTAs without rows: they must not start copies that nothing waits for
+  if ((int)blockIdx.y * Cfg::kRows >= ch.nrows) return;
   for (int w = tid; w < R * kW; w += Cfg::kThreads)
     cp_async_16(LT + (w / kW) * kLd + 4 * (w % kW), L + 4 * w, 16);
   for (int s0 = blockIdx.y * Cfg::kRows; s0 < ch.nrows; s0 += gridDim.y * Cfg::kRows) {

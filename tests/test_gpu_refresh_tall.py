@@ -45,10 +45,11 @@ def test_tall_panels_match_oracle(lib, gpu, r):
     one.close()
 
 
-@pytest.mark.parametrize("r", [16, 32, 64])
+@pytest.mark.parametrize("r", [16, 32, 64, 128])
 def test_many_chunks_have_the_bits_of_few(lib, gpu, r):
-    """More than 608 chunks (several per CTA, the last CTA's incomplete, panels of one and of two
-    chunks): each panel has the bits it has in a context of its own."""
+    """More than 608 chunks (at r < 128 several per CTA, the last CTA's incomplete; panels of one and
+    of two chunks, the second of 16 rows, so that most of the CTAs its slices are dealt to have
+    none): each panel has the bits it has in a context of its own."""
     from paper_2608_15665_gb300.schedule import SubZeroPlus
     n = [(4 * r + 1, 4 * r + 37)] * 306 + [(1040, 4 * r)]
     weights = [torch.zeros(a, (b + 7) // 8 * 8, dtype=torch.bfloat16, device=gpu)[:, :b] for a, b in n]
