@@ -1193,7 +1193,7 @@ zo_status zo_linear_perturbed(zo_ctx* c, int32_t mat, const void* X, int64_t T, 
   const zo::LinearFewPlan few = c->linear_tile == 0 ? zo::linear_few_plan(T, m, n, r, c->sms)
                                                     : zo::LinearFewPlan{};
   if (few.ctas > 0) {
-    const zo_status ws = linear_workspace(c, T, T * r);
+    const zo_status ws = linear_workspace(c, T, 0);
     if (ws != ZO_OK) return ws;
     CUtensorMap tm_x{}, tm_xs{}, tm_w{}, tm_pk{}, tm_s{}, tm_u{};
     void* x = const_cast<void*>(X);
@@ -1254,7 +1254,7 @@ zo_status zo_linear_perturbed(zo_ctx* c, int32_t mat, const void* X, int64_t T, 
   } else {
     zo::linear_s_split(T, n, c->sms, &k_split, &k_chunk);
   }
-  const int64_t part = (int64_t)k_split * T * r;
+  const int64_t part = k_split * ((T + 127) / 128 * 128) * r;   // as the token capacity grows
   const zo_status st = linear_workspace(c, T, part);
   if (st != ZO_OK) return st;
   const bool narrow_y = pair_n == 0 && zo::linear_y_tile_cols(tiling) % 64 != 0;
