@@ -254,8 +254,10 @@ ZO_API zo_status zo_mezo_perturb(zo_ctx* ctx, uint32_t t, float coef);
  *   accumulation; the rank-r term carries the bf16 hi/lo split's ~2^-16 relative error;
  *   Y is rounded to bf16 once.  W_i is read, never written.  Asynchronous; device errors
  *   go to the status word.  The GEMM's tiling follows ZO_OPTION_LINEAR_TILE (the tilings
- *   of one family give the same Y bits); the context keeps an S workspace sized for the most tokens
- *   seen so far, and a call with more synchronises the stream to grow it.
+ *   of one family give the same Y bits); the context keeps an S workspace sized for the most
+ *   tokens seen so far, and a call that needs more synchronises the stream to grow it, which
+ *   is an error under stream capture.  A call captured into a graph may be replayed on other
+ *   contents of X until a later call grows the workspace.
  */
 ZO_API zo_status zo_linear_prepare(zo_ctx* ctx, uint32_t t, int32_t qa, float ca, int32_t qb,
                                    float cb, float eps);

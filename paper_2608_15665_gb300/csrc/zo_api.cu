@@ -1146,17 +1146,20 @@ zo_status linear_workspace(zo_ctx* c, int64_t T, int64_t part) {
   return ZO_OK;
 }
 
-// The epoch of the next launch that counts in the row-block flags and counters.
+// The epoch of the next launch that counts in the row-block flags and counters.  A launch
+// captured into a graph keeps its epoch in every replay, whose flags the replay before has set:
+// it takes the last epoch, which no live launch has, and the graph zeroes the flags before it.
 zo_status linear_epoch(zo_ctx* c, uint32_t* epoch) {
-  if (c->lin_epoch + 1 >= zo::kLinearPairEpochs) {
-    // the epochs start again: no flag or counter may hold an old call's
-    ZO_CUDA(cudaMemsetAsync(c->d_s_flags, 0,
-                            sizeof(uint32_t) * s_flag_words(c),
-                            c->stream),
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(c->stream, &cap) != cudaSuccess) cudaGetLastError();
+  const bool captured = cap == cudaStreamCaptureStatusActive;
+  // live epochs that start again: no flag or counter may hold an old call's
+  const bool wrap = !captured && c->lin_epoch + 2 >= zo::kLinearPairEpochs;
+  if (captured || wrap)
+    ZO_CUDA(cudaMemsetAsync(c->d_s_flags, 0, sizeof(uint32_t) * s_flag_words(c), c->stream),
             "zero S row-block counters");
-    c->lin_epoch = 0;
-  }
-  *epoch = ++c->lin_epoch;
+  if (wrap) c->lin_epoch = 0;
+  *epoch = captured ? zo::kLinearPairEpochs - 1 : ++c->lin_epoch;
   return ZO_OK;
 }
 

@@ -229,8 +229,9 @@ int32_t linear_pair_tiling(int64_t T, int64_t m, int64_t n, int32_t r, int32_t n
 // swizzle), tm_pk over P_K (box 64 x r), tm_ps over P_K (box 64 x s_cols / 2; any box when
 // n_contrib = 0).  s_part: s_split x T x r floats (s_split > 1).  s_count:
 // kLinearPairCounters counters per 256 rows of X (zero before the first call), epoch:
-// 1 .. kLinearPairEpochs - 1, a new one per call (the counters of a launch cut short by a
-// wait timeout must be zeroed before the epochs start again).  inject_wait (test hook):
+// 1 .. kLinearPairEpochs - 1, one that no counter holds: a new one per call, or zeroed counters
+// (so too before the epochs start again after a launch cut short by a wait timeout).
+// inject_wait (test hook):
 // the Y tiles wait for a count that never comes, with the short test limit; the launch
 // then reports kDevTimeout.
 cudaError_t launch_linear_pair(const CUtensorMap& tm_x, const CUtensorMap& tm_w,
