@@ -862,7 +862,7 @@ zo_status zo_refresh(zo_ctx* c, uint32_t refresh_idx, int32_t reset_moments) {
   if (c->n_cq_panels > 0) {
     ZO_CUDA(zo::launch_cholqr(c->d_cq_panels, c->n_cq_panels, c->d_cq_chunks, c->n_cq_chunks,
                               c->d_cq_partial, c->d_cq_linv, c->r, c->seed, refresh_idx,
-                              c->d_status, c->stream),
+                              c->sms, c->d_status, c->stream),
             "refresh CholeskyQR2 kernels");
     c->launches += 6;
   }

@@ -471,7 +471,7 @@ size_t chol_smem() { return sizeof(float) * R * (R + 1); }
 template <int R>
 cudaError_t run_cholqr_r(const CqPanel* d_panels, int32_t n_panels, const CqChunk* d_chunks,
                          int32_t n_chunks, float* d_partial, float* d_linv, uint64_t seed,
-                         uint32_t refresh_idx, uint32_t* d_status, cudaStream_t s) {
+                         uint32_t refresh_idx, int32_t sms, uint32_t* d_status, cudaStream_t s) {
   cudaError_t e = cudaFuncSetAttribute(cq_chol_kernel<R>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)chol_smem<R>());
   if (e == cudaSuccess)
@@ -479,15 +479,23 @@ cudaError_t run_cholqr_r(const CqPanel* d_panels, int32_t n_panels, const CqChun
                              (int)Apply<R>::kSmem);
   if (e != cudaSuccess) return e;
   constexpr int kT = R == 16 ? 2 : 4, kG = R == 128 ? 1 : 2;
-  // fewer than four chunks per SM: a CTA each (as ordinary launches; two per CTA: one 4096 x 4096
-  // matrix at r = 64 246 us a refresh instead of 190, one 7B layer at r = 32 160 instead of 141)
-  const bool few = n_chunks < 608;
-  // Few chunks: launches that wait for their predecessor and overlap its tail (one 4096 x 4096
-  // matrix 185 -> 169 us at r = 64, 74 -> 59 at r = 16).  Not at r = 128, where the next kernel's
-  // large CTAs take the SM from this one's (one 7B layer: 467 -> 512 us).
+  // Fewer than four chunks per SM: a CTA of the Gram kernels each, and launches that wait for
+  // their predecessor and overlap its tail; else kG chunks per CTA and ordinary launches.  A
+  // refresh in us on 152 SMs, this way / the other, of 4096 x 1024 matrices:
+  //   chunks     80       320        610        960         1280         2560         3840
+  //   r = 16   67 / 111  104 / 132  143 / 165  193 / 214   253 / 268    471 / 490    687 / 677
+  //   r = 32  133 / 157  206 / 219  300 / 314  443 / 432   541 / 539    989 / 962   1472 / 1385
+  //   r = 64  194 / 266  376 / 458  634 / 686  899 / 957  1126 / 1196  2117 / 2172  3153 / 3139
+  // (whole layers of the 1.3B, 7B and 32B sets alike).  The line is r = 32's; at r = 16 and 64,
+  // where it leaves 2 to 15% between 608 and some 2500 chunks, it is kept for one rule.
+  const bool few = n_chunks < 4 * sms;
+  // Not dependent at r = 128, where the next kernel's large CTAs take the SM from this one's (one
+  // 7B layer: 467 -> 512 us).
   const bool dep = few && R < 128;
-  // CTAs per chunk: one tile each; at r = 128, two 64-row tiles of 16 where chunks are many, for
-  // L^-1's 64 KB (8 layers of the 7B set: 1.82 ms, one per CTA 1.84; one layer 476 and 467 us)
+  // CTAs per chunk of the triangular product.  r < 128: eight, a 128-row tile each.  r = 128: two
+  // 64-row tiles each, four where chunks are many, for the 64 KB of L^-1 that each CTA copies
+  // (4096 x 1024 matrices, eight / four CTAs: 469 / 488 us at 80 chunks, 1187 / 1188 at 320, 1658 /
+  // 1636 at 480, 2022 / 2005 at 610, 3839 / 3755 at 1280).
   const int n_split = R < 128 || few ? 8 : 4;
   // first Cholesky QR: Omega -> Q1; second: Q1 -> Q; both in the panels
   for (int round = 0; round < 2; ++round) {
@@ -514,13 +522,14 @@ bool cholqr_supported(int32_t r) { return r == 16 || r == 32 || r == 64 || r == 
 
 cudaError_t launch_cholqr(const CqPanel* d_panels, int32_t n_panels, const CqChunk* d_chunks,
                           int32_t n_chunks, float* d_partial, float* d_linv, int32_t r,
-                          uint64_t seed, uint32_t refresh_idx, uint32_t* d_status, cudaStream_t s) {
+                          uint64_t seed, uint32_t refresh_idx, int32_t sms, uint32_t* d_status,
+                          cudaStream_t s) {
   if (n_panels <= 0) return cudaSuccess;
   switch (r) {
-    case 16: return run_cholqr_r<16>(d_panels, n_panels, d_chunks, n_chunks, d_partial, d_linv, seed, refresh_idx, d_status, s);
-    case 32: return run_cholqr_r<32>(d_panels, n_panels, d_chunks, n_chunks, d_partial, d_linv, seed, refresh_idx, d_status, s);
-    case 64: return run_cholqr_r<64>(d_panels, n_panels, d_chunks, n_chunks, d_partial, d_linv, seed, refresh_idx, d_status, s);
-    case 128: return run_cholqr_r<128>(d_panels, n_panels, d_chunks, n_chunks, d_partial, d_linv, seed, refresh_idx, d_status, s);
+    case 16: return run_cholqr_r<16>(d_panels, n_panels, d_chunks, n_chunks, d_partial, d_linv, seed, refresh_idx, sms, d_status, s);
+    case 32: return run_cholqr_r<32>(d_panels, n_panels, d_chunks, n_chunks, d_partial, d_linv, seed, refresh_idx, sms, d_status, s);
+    case 64: return run_cholqr_r<64>(d_panels, n_panels, d_chunks, n_chunks, d_partial, d_linv, seed, refresh_idx, sms, d_status, s);
+    case 128: return run_cholqr_r<128>(d_panels, n_panels, d_chunks, n_chunks, d_partial, d_linv, seed, refresh_idx, sms, d_status, s);
     default: return cudaErrorInvalidValue;
   }
 }

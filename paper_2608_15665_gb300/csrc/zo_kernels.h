@@ -291,7 +291,8 @@ bool cholqr_supported(int32_t r);
 // floats (its lower blocks are written), d_linv: n_panels x r x r floats (L^-1 transposed).
 cudaError_t launch_cholqr(const CqPanel* d_panels, int32_t n_panels, const CqChunk* d_chunks,
                           int32_t n_chunks, float* d_partial, float* d_linv, int32_t r,
-                          uint64_t seed, uint32_t refresh_idx, uint32_t* d_status, cudaStream_t s);
+                          uint64_t seed, uint32_t refresh_idx, int32_t sms, uint32_t* d_status,
+                          cudaStream_t s);
 
 // ---- refresh of fp32 weights at r = 4 and 8, panel in registers (zo_cholqr_small.cu) ---
 // CTAs (a cluster of 1, 2, 4 or 8) that hold a tall panel, 0 if it is not for this kernel;
