@@ -44,16 +44,16 @@ TRAFFIC_BY_SOURCE = {
     # code hash of the kernel that runs (comments ignored) -> dram read + write bytes of one
     # launch, from an ncu capture on a small case of the same workload, scaled by weights
     # profiles/wpass_tc_r32_llama7b_2layers.md: 1.5776 GB on the 2-layer subset, x16.0
-    ("32b0dddb3786330a", "llama7b_bf16_r32"): 25.24e9,
+    ("a008d98398cee6e8", "llama7b_bf16_r32"): 25.24e9,
     # profiles/wpass_pair_r128_llama7b_2layers.md: 1.6395 GB on the 2-layer subset, x16.0
-    ("d1d9e6f8246f6b1f", "llama7b_bf16_r128_q99"): 26.23e9,
+    ("dcdb8ae8f4f41a1c", "llama7b_bf16_r128_q99"): 26.23e9,
     # profiles/wpass_tmem_r64_dense32b_1layer.md: 1.9265 GB on the 1-layer subset, x64.0
-    ("2e37b0bf937bfe68", "dense32b_bf16_r64"): 123.30e9,
+    ("76ab4e4bc4fa75c2", "dense32b_bf16_r64"): 123.30e9,
 }
 # thread instructions per weight of the full-space SPSA kernel (ncu), keyed by source hash
 INSTR_PER_WEIGHT_BY_SOURCE = {
     # profiles/mezo_kernel_llama7b_2layers.md: 482.6 M warp instructions x 32 / 404.75 M weights
-    "59503d8e1c27879d": 38.2,
+    "5871db0ab409c6bb": 38.2,
 }
 
 
@@ -113,15 +113,25 @@ def _code_hash(names):
     return h.hexdigest()[:16]
 
 
+def kernel_sources(name):
+    """A kernel file and the headers it includes, directly or through one another."""
+    names, todo = [], [name]
+    while todo:
+        name = todo.pop()
+        path = os.path.join(ROOT, "paper_2608_15665_gb300", "csrc", name)
+        if name in names or not os.path.exists(path):
+            continue
+        names.append(name)
+        todo += re.findall(r'^\s*#include "([^"/]+)"', open(path, encoding="utf-8").read(), flags=re.M)
+    return names[:1] + sorted(names[1:])
+
+
 def kernel_source_hash(r=32):
     """Code hash of the tensor-core weight-pass kernel that runs at rank r (r <= 32:
-    zo_wpass_tc.cu, r = 64: zo_wpass_tmem.cu, r = 128: zo_wpass_pair.cu) and the headers
-    it includes."""
+    zo_wpass_tc.cu, r = 64: zo_wpass_tmem.cu, r = 128: zo_wpass_pair.cu) and every header
+    that is compiled into it."""
     kernel = "zo_wpass_tc.cu" if r <= 32 else "zo_wpass_tmem.cu" if r == 64 else "zo_wpass_pair.cu"
-    headers = ("zo_tc_common.cuh", "zo_sm100.cuh", "zo_device.cuh")
-    if r == 128:
-        headers += ("zo_cluster.cuh",)
-    return _code_hash((kernel,) + headers)
+    return _code_hash(kernel_sources(kernel))
 
 
 def subset(wl, layers):
@@ -138,7 +148,7 @@ def subset(wl, layers):
 
 
 def mezo_source_hash():
-    return _code_hash(("zo_mezo.cu", "zo_device.cuh"))
+    return _code_hash(kernel_sources("zo_mezo.cu"))
 
 
 # --------------------------------------------------------------------------- clocks

@@ -4,6 +4,7 @@ hash that keys the ncu-derived traffic, and the layer subsets used for profiling
 
 import json
 import os
+import shutil
 import subprocess
 import sys
 
@@ -108,6 +109,31 @@ def test_code_hash_ignores_comments_and_spacing(tmp_path, monkeypatch):
     assert bench._code_hash(["k.cu"]) == h0
     (csrc / "k.cu").write_text("int f(int x) { return x + 2; }\n")
     assert bench._code_hash(["k.cu"]) != h0
+
+
+@pytest.mark.parametrize("header, of", [
+    ("zo_launch.cuh", {16, 32, 64, 128}),          # the dependent launches' wait
+    ("zo_sm100.cuh", {16, 32, 64, 128}),
+    ("zo_cluster.cuh", {128}),
+    ("zo_fma_common.cuh", {"mezo"}),               # the tile lookup, vectors of W, rounding
+    ("zo_device.cuh", {16, 32, 64, 128, "mezo"}),
+])
+def test_source_hashes_cover_every_included_header(header, of, tmp_path, monkeypatch):
+    """An edit of a header changes the hash of exactly the kernels that are compiled with it, so
+    that counters of the old code are not reported as theirs."""
+    import bench
+    csrc = tmp_path / "paper_2608_15665_gb300" / "csrc"
+    shutil.copytree(os.path.join(ROOT, "paper_2608_15665_gb300", "csrc"), csrc)
+
+    def hashes():
+        return {**{r: bench.kernel_source_hash(r) for r in (16, 32, 64, 128)},
+                "mezo": bench.mezo_source_hash()}
+
+    monkeypatch.setattr(bench, "ROOT", str(tmp_path))
+    before = hashes()
+    (csrc / header).write_text((csrc / header).read_text() + "\nconstexpr int kEdited = 1;\n")
+    after = hashes()
+    assert {k for k in before if before[k] != after[k]} == of
 
 
 def test_layer_subsets_keep_the_shapes_and_zero_init_of_their_layers():
