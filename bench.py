@@ -134,6 +134,16 @@ def kernel_source_hash(r=32):
     return _code_hash(kernel_sources(kernel))
 
 
+def wpass_kernel_name(path, r, single_sm=False):
+    """The weight-pass kernel of a path as zo_wpass_path reports it, at rank r.  On full tiles
+    of the FMA path at r in {4, 8}, small sets take their perturbations by the one-launch kernel
+    and the step's update by the other."""
+    return {1: "wpass_gemm" if r >= 16 else "wpass_fma_fused / wpass_gemm",
+            2: ("wpass_tmem" if single_sm else "wpass_pair") if r == 128
+            else "wpass_tmem" if r == 64 else "wpass_tc",
+            3: "wpass_narrow"}.get(path, "?")
+
+
 def subset(wl, layers):
     """The first `layers` layers of a workload (its matrices repeat per layer)."""
     if not layers:
@@ -537,10 +547,7 @@ def run_ours(args):
         "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                      "frac": achieved / peak, "peak_kind": peak_kind,
                      "traffic": TRAFFIC_BY_SOURCE.get((src, wl.name)),
-                     "kernel": {1: "wpass_fma",
-                                2: ("wpass_tmem" if args.single_sm else "wpass_pair") if wl.r == 128
-                                else "wpass_tmem" if wl.r == 64 else "wpass_tc",
-                                3: "wpass_narrow"}.get(path, "?"),
+                     "kernel": wpass_kernel_name(path, wl.r, args.single_sm),
                      "algorithmic_bytes_per_launch": bytes_pass,
                      "avg_launch_ms": avg_launch_s * 1e3, "launches_timed": wpass_n},
         "clocks": clk,
@@ -657,8 +664,7 @@ def secondary_weight_pass(dev, local, peak, name, K):
     step_ms = window_ms / K + refresh_ms / wl.F
     return {"workload": wl.name, "matrices": wl.n_mats, "params": wl.params, "r": wl.r, "q": wl.q,
             "passes_per_step": 2 * wl.q + 1, "refresh_every": wl.F, "steps_timed": K,
-            "kernel": {2: "wpass_pair" if wl.r == 128 else "wpass_tmem" if wl.r == 64
-                       else "wpass_tc", 1: "wpass_fma"}.get(path, "?"),
+            "kernel": wpass_kernel_name(path, wl.r),
             "avg_launch_ms": avg_s * 1e3, "launches_timed": wpass_n,
             "algorithmic_bytes_per_launch": wl.bytes_per_pass(),
             "achieved_gbs": achieved, "peak_gbs": peak, "frac": achieved / peak,

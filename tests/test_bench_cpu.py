@@ -136,6 +136,19 @@ def test_source_hashes_cover_every_included_header(header, of, tmp_path, monkeyp
     assert {k for k in before if before[k] != after[k]} == of
 
 
+def test_weight_pass_kernels_are_named_as_they_exist():
+    """Every name that the roofline can carry is a kernel of the library."""
+    import bench
+    csrc = os.path.join(ROOT, "paper_2608_15665_gb300", "csrc")
+    code = "".join(open(os.path.join(csrc, f), encoding="utf-8").read()
+                   for f in os.listdir(csrc) if f.endswith(".cu"))
+    for path in (1, 2, 3):
+        for r in (4, 8, 16, 32, 64, 128):
+            for name in bench.wpass_kernel_name(path, r).split(" / "):
+                assert f"\n{name}_kernel(" in code or f" {name}_kernel(" in code, name
+    assert bench.wpass_kernel_name(2, 128, single_sm=True) == "wpass_tmem"
+
+
 def test_layer_subsets_keep_the_shapes_and_zero_init_of_their_layers():
     import bench
     from paper_2608_15665_gb300 import workloads
