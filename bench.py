@@ -44,16 +44,16 @@ TRAFFIC_BY_SOURCE = {
     # code hash of the kernel that runs (comments ignored) -> dram read + write bytes of one
     # launch, from an ncu capture on a small case of the same workload, scaled by weights
     # profiles/wpass_tc_r32_llama7b_2layers.md: 1.5776 GB on the 2-layer subset, x16.0
-    ("a008d98398cee6e8", "llama7b_bf16_r32"): 25.24e9,
+    ("c1df6315339b03e5", "llama7b_bf16_r32"): 25.24e9,
     # profiles/wpass_pair_r128_llama7b_2layers.md: 1.6395 GB on the 2-layer subset, x16.0
-    ("dcdb8ae8f4f41a1c", "llama7b_bf16_r128_q99"): 26.23e9,
+    ("8a2d86063f09c61b", "llama7b_bf16_r128_q99"): 26.23e9,
     # profiles/wpass_tmem_r64_dense32b_1layer.md: 1.9265 GB on the 1-layer subset, x64.0
-    ("76ab4e4bc4fa75c2", "dense32b_bf16_r64"): 123.30e9,
+    ("8c8de09c3a872d01", "dense32b_bf16_r64"): 123.30e9,
 }
 # thread instructions per weight of the full-space SPSA kernel (ncu), keyed by source hash
 INSTR_PER_WEIGHT_BY_SOURCE = {
     # profiles/mezo_kernel_llama7b_2layers.md: 482.6 M warp instructions x 32 / 404.75 M weights
-    "5871db0ab409c6bb": 38.2,
+    "fd0f60b263432f6f": 38.2,
 }
 
 

@@ -22,7 +22,7 @@ enum DeviceStatus : uint32_t {
   kDevNotPosDef = 4, // refresh: a Gram matrix had a non-positive Cholesky pivot
 };
 
-// Two fp32 operations (each lane rounded to nearest, as fmaf, * and +) in one instruction.
+// Two fp32 operations (each lane rounded to nearest, as fmaf and *) in one instruction.
 __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {
   float2 d;
   asm("{\n\t.reg .b64 a, b, c, d;\n\t"
@@ -37,15 +37,6 @@ __device__ __forceinline__ float2 mul2(float2 a, float2 b) {
   asm("{\n\t.reg .b64 a, b, d;\n\t"
       "mov.b64 a, {%2, %3};\n\tmov.b64 b, {%4, %5};\n\t"
       "mul.rn.f32x2 d, a, b;\n\tmov.b64 {%0, %1}, d;\n\t}"
-      : "=f"(d.x), "=f"(d.y)
-      : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
-  return d;
-}
-__device__ __forceinline__ float2 add2(float2 a, float2 b) {
-  float2 d;
-  asm("{\n\t.reg .b64 a, b, d;\n\t"
-      "mov.b64 a, {%2, %3};\n\tmov.b64 b, {%4, %5};\n\t"
-      "add.rn.f32x2 d, a, b;\n\tmov.b64 {%0, %1}, d;\n\t}"
       : "=f"(d.x), "=f"(d.y)
       : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
   return d;
@@ -85,28 +76,6 @@ __device__ __forceinline__ float u01(uint32_t x) {
   return __uint2float_rn((x >> 8) + 1u) * 5.9604644775390625e-08f;
 }
 
-// The transform below runs on one value at a time (float) or on packed pairs (float2); both
-// round every operation alike, so they give the same bits.
-__device__ __forceinline__ float vfma(float a, float b, float c) { return fmaf(a, b, c); }
-__device__ __forceinline__ float2 vfma(float2 a, float2 b, float2 c) { return fma2(a, b, c); }
-__device__ __forceinline__ float vmul(float a, float b) { return __fmul_rn(a, b); }
-__device__ __forceinline__ float2 vmul(float2 a, float2 b) { return mul2(a, b); }
-__device__ __forceinline__ float vadd(float a, float b) { return __fadd_rn(a, b); }
-__device__ __forceinline__ float2 vadd(float2 a, float2 b) { return add2(a, b); }
-template <typename V> struct Lanes;
-template <> struct Lanes<float> {
-  static constexpr int N = 1;
-  static __device__ __forceinline__ float all(float x) { return x; }
-  static __device__ __forceinline__ float from(const float* x) { return x[0]; }
-  static __device__ __forceinline__ void to(float v, float* x) { x[0] = v; }
-};
-template <> struct Lanes<float2> {
-  static constexpr int N = 2;
-  static __device__ __forceinline__ float2 all(float x) { return make_float2(x, x); }
-  static __device__ __forceinline__ float2 from(const float* x) { return make_float2(x[0], x[1]); }
-  static __device__ __forceinline__ void to(float2 v, float* x) { x[0] = v.x; x[1] = v.y; }
-};
-
 // Box-Muller on kV vectors of word pairs (xa, xb), u = ((x >> 8) + 1) 2^-24 in (0, 1]:
 // rad cos 2 pi ub = nr c and rad sin 2 pi ub = nr s with nr = -rad = -sqrt(-2 ln ua).  The
 // uniforms are integers over 2^24, so both functions reduce their arguments exactly, in
@@ -121,90 +90,86 @@ template <> struct Lanes<float2> {
 //    its error in q, cos = 1 + t^2 p(t^2) (2.5e-9 and 6e-11); the quadrant swaps and negates.
 // Over all 2^24 uniforms (double precision): radius within 3.5e-7 (rms 4.05e-8), cos and sin
 // within 6.1e-8, no further off than logf, sqrtf and sincospif.
-template <int kV, typename V>
-__device__ __forceinline__ void box_muller_parts(const uint32_t (&xa)[kV * Lanes<V>::N],
-                                                 const uint32_t (&xb)[kV * Lanes<V>::N],
-                                                 V (&nr)[kV], V (&zc)[kV], V (&zs)[kV]) {
-  using LN = Lanes<V>;
-  constexpr int kL = LN::N, kN = kV * kL;
+template <int kV>
+__device__ __forceinline__ void box_muller_parts(const uint32_t (&xa)[2 * kV],
+                                                 const uint32_t (&xb)[2 * kV], float2 (&nr)[kV],
+                                                 float2 (&zc)[kV], float2 (&zs)[kV]) {
+  auto all = [](float x) { return make_float2(x, x); };
   {
-    V g[kV], e[kV], P[kV];
+    float2 g[kV], e[kV], P[kV];
 #pragma unroll
     for (int v = 0; v < kV; ++v) {
-      float m[kL], x[kL];
+      float m[2], x[2];
 #pragma unroll
-      for (int l = 0; l < kL; ++l) {
-        const int k = __float_as_int(__uint2float_rn((xa[v * kL + l] >> 8) + 1u));
+      for (int l = 0; l < 2; ++l) {
+        const int k = __float_as_int(__uint2float_rn((xa[v * 2 + l] >> 8) + 1u));
         const int ex = (k - 0x4b2aaaab) & (int)0xff800000;     // (e - 24) 2^23
         m[l] = __int_as_float(k - ex - 0x0c000000);
         x[l] = __int2float_rn(ex);
       }
-      g[v] = vfma(LN::from(m), LN::all(2.0f), LN::all(-2.0f));
-      e[v] = LN::from(x);
+      g[v] = fma2(make_float2(m[0], m[1]), all(2.0f), all(-2.0f));
+      e[v] = make_float2(x[0], x[1]);
     }
     constexpr float kP[9] = {-0x1p-2f,        0x1.55550cp-4f,  -0x1.fffe5ep-6f,
                              0x1.99ce34p-7f,  -0x1.55b7ecp-8f, 0x1.1ef264p-9f,
                              -0x1.f03bdcp-11f, 0x1.1defc4p-11f, -0x1.0e2acep-12f};
 #pragma unroll
-    for (int v = 0; v < kV; ++v) P[v] = LN::all(kP[8]);
+    for (int v = 0; v < kV; ++v) P[v] = all(kP[8]);
 #pragma unroll
     for (int i = 7; i >= 0; --i)
 #pragma unroll
-      for (int v = 0; v < kV; ++v) P[v] = vfma(P[v], g[v], LN::all(kP[i]));
+      for (int v = 0; v < kV; ++v) P[v] = fma2(P[v], g[v], all(kP[i]));
 #pragma unroll
     for (int v = 0; v < kV; ++v) {
-      V nl = vfma(vmul(g[v], g[v]), P[v], g[v]);
-      nl = vfma(e[v], LN::all(0x1.62e430p-23f), nl);           // 2 ln u
-      float x[kL], y[kL];
-      LN::to(nl, x);
-#pragma unroll
-      for (int l = 0; l < kL; ++l)
-        asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y[l]) : "f"(fmaxf(-x[l], 1e-30f)));
-      const V ns = vmul(nl, LN::from(y));
-      nr[v] = vfma(vfma(ns, ns, nl), vmul(LN::from(y), LN::all(0.5f)), ns);
+      float2 nl = fma2(mul2(g[v], g[v]), P[v], g[v]);
+      nl = fma2(e[v], all(0x1.62e430p-23f), nl);               // 2 ln u
+      float2 y;
+      asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y.x) : "f"(fmaxf(-nl.x, 1e-30f)));
+      asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y.y) : "f"(fmaxf(-nl.y, 1e-30f)));
+      const float2 ns = mul2(nl, y);
+      nr[v] = fma2(fma2(ns, ns, nl), mul2(y, all(0.5f)), ns);
     }
   }
-  uint32_t qd[kN];                                             // (k + 2^21) 2^8
-  V t[kV], w[kV], sn[kV], cs[kV];
+  uint32_t qd[2 * kV];                                         // (k + 2^21) 2^8
+  float2 t[kV], w[kV], sn[kV], cs[kV];
 #pragma unroll
   for (int v = 0; v < kV; ++v) {
-    float j[kL];
+    float j[2];
 #pragma unroll
-    for (int l = 0; l < kL; ++l) {
-      qd[v * kL + l] = xb[v * kL + l] + 0x20000100u;
-      j[l] = __uint_as_float(((qd[v * kL + l] >> 8) & 0x3fffffu) | 0x4b000000u);   // 2^23 + j
+    for (int l = 0; l < 2; ++l) {
+      qd[v * 2 + l] = xb[v * 2 + l] + 0x20000100u;
+      j[l] = __uint_as_float(((qd[v * 2 + l] >> 8) & 0x3fffffu) | 0x4b000000u);   // 2^23 + j
     }
-    t[v] = vfma(LN::from(j), LN::all(0x1p-21f), LN::all(-5.0f));
-    w[v] = vmul(t[v], t[v]);
+    t[v] = fma2(make_float2(j[0], j[1]), all(0x1p-21f), all(-5.0f));
+    w[v] = mul2(t[v], t[v]);
   }
   constexpr float kS[4] = {-0x1.a0f38ap-26f, -0x1.4abbbap-4f, 0x1.465ee8p-9f, -0x1.2da132p-15f};
   constexpr float kC[4] = {-0x1.3bd3ccp-2f, 0x1.03c1e2p-6f, -0x1.55c752p-12f, 0x1.da30fap-19f};
 #pragma unroll
-  for (int v = 0; v < kV; ++v) { sn[v] = LN::all(kS[3]); cs[v] = LN::all(kC[3]); }
+  for (int v = 0; v < kV; ++v) { sn[v] = all(kS[3]); cs[v] = all(kC[3]); }
 #pragma unroll
   for (int i = 2; i >= 0; --i)
 #pragma unroll
     for (int v = 0; v < kV; ++v) {
-      sn[v] = vfma(w[v], sn[v], LN::all(kS[i]));
-      cs[v] = vfma(w[v], cs[v], LN::all(kC[i]));
+      sn[v] = fma2(w[v], sn[v], all(kS[i]));
+      cs[v] = fma2(w[v], cs[v], all(kC[i]));
     }
 #pragma unroll
   for (int v = 0; v < kV; ++v) {
-    sn[v] = vfma(t[v], LN::all(0x1.921fb6p-1f), vmul(t[v], sn[v]));
-    cs[v] = vfma(w[v], cs[v], LN::all(1.0f));
-    float a[kL], b[kL], c[kL], s[kL];
-    LN::to(cs[v], a);
-    LN::to(sn[v], b);
+    sn[v] = fma2(t[v], all(0x1.921fb6p-1f), mul2(t[v], sn[v]));
+    cs[v] = fma2(w[v], cs[v], all(1.0f));
+    const float a[2] = {cs[v].x, cs[v].y}, b[2] = {sn[v].x, sn[v].y};
+    float c[2], s[2];
 #pragma unroll
-    for (int l = 0; l < kL; ++l) {
-      const uint32_t q = qd[v * kL + l];
+    for (int l = 0; l < 2; ++l) {
+      const uint32_t q = qd[v * 2 + l];
       const bool odd = (q & 0x40000000u) != 0;
       // cos is negative in quadrants 1 and 2, sin in 2 and 3; both negated, as nr is -rad
       c[l] = __uint_as_float(__float_as_uint(odd ? b[l] : a[l]) ^ ((q + 0xc0000000u) & 0x80000000u));
       s[l] = __uint_as_float(__float_as_uint(odd ? a[l] : b[l]) ^ (~q & 0x80000000u));
     }
-    zc[v] = LN::from(c);
-    zs[v] = LN::from(s);
+    zc[v] = make_float2(c[0], c[1]);
+    zs[v] = make_float2(s[0], s[1]);
   }
 }
 
@@ -234,7 +199,7 @@ __device__ __forceinline__ float4 normal4_packed(uint64_t seed, uint32_t c4, uin
                                 static_cast<uint32_t>(seed >> 32));
   const uint32_t a[2] = {w.x, w.z}, b[2] = {w.y, w.w};
   float2 nr[1], c[1], s[1];
-  box_muller_parts<1, float2>(a, b, nr, c, s);
+  box_muller_parts<1>(a, b, nr, c, s);
   c[0] = mul2(nr[0], c[0]);
   s[0] = mul2(nr[0], s[0]);
   return make_float4(c[0].x, s[0].x, c[0].y, s[0].y);

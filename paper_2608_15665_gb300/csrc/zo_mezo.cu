@@ -92,7 +92,7 @@ __device__ __forceinline__ void mezo_tile(const MatDesc& md, int64_t local, cons
         xa[p] = x.x; xb[p] = x.y; xa[p + 1] = x.z; xb[p + 1] = x.w;
       }
     float2 nr[kN / 2], zc[kN / 2], zs[kN / 2];
-    box_muller_parts<kN / 2, float2>(xa, xb, nr, zc, zs);
+    box_muller_parts<kN / 2>(xa, xb, nr, zc, zs);
 #pragma unroll
     for (int p = 0; p < kN / 2; ++p) {
       zc[p] = mul2(nr[p], zc[p]);

@@ -18,7 +18,7 @@
 __device__ float2 normals(uint32_t xa, uint32_t xb) {
   const uint32_t a[2] = {xa, xa}, b[2] = {xb, xb};
   float2 nr[1], c[1], s[1];
-  zo::box_muller_parts<1, float2>(a, b, nr, c, s);
+  zo::box_muller_parts<1>(a, b, nr, c, s);
   const float2 z0 = zo::mul2(nr[0], c[0]), z1 = zo::mul2(nr[0], s[0]);
   return z0.x == z0.y && z1.x == z1.y ? make_float2(z0.x, z1.x) : make_float2(nanf(""), nanf(""));
 }
