@@ -79,15 +79,21 @@ __device__ __forceinline__ float u01(uint32_t x) {
 // Box-Muller on kV vectors of word pairs (xa, xb), u = ((x >> 8) + 1) 2^-24 in (0, 1]:
 // rad cos 2 pi ub = nr c and rad sin 2 pi ub = nr s with nr = -rad = -sqrt(-2 ln ua).  The
 // uniforms are integers over 2^24, so both functions reduce their arguments exactly, in
-// integers; the polynomials are minimax fits whose coefficients are rounded from the lowest
-// order on, the rest refitted:
-//  * ln: k = u 2^24 = m 2^e with m in [2/3, 4/3), g = 2 m - 2 exact, 2 ln u = (e - 24) 2 ln 2
-//    + g + g^2 P(g), P of degree 8 (5.0e-9 of the result).
+// integers:
+//  * ln: k = u 2^24 = m 2^e with m near 1 (the reduction of Cody and Waite, Software Manual for
+//    the Elementary Functions, 1980), in [2/3, 4/3), where m - 1 reaches as far to either side:
+//    k's bits less those of (2/3) 2^24 hold e - 24 above the mantissa.  g = 2 m - 2 exact,
+//    2 ln u = (e - 24) 2 ln 2 + g + g^2 P(g), P of degree 8.
 //  * sqrt of x = -2 ln u: the hardware's reciprocal square root y, s = x y, and one Newton
-//    step s + (x - s^2) y / 2, all with the sign turned; u = 1 gives 0.
+//    step by the residual, s + (x - s^2) y / 2 (Markstein, IBM J. Res. Dev. 34, 1990), all with
+//    the sign turned; u = 1 gives 0.
 //  * cos, sin: k + 2^21 = quadrant 2^22 + j, the angle inside the quadrant (pi/4) t with
 //    t = (j - 2^21) 2^-21 exact in [-1, 1); sin = t s0 + t q(t^2) with s0 the fp32 pi/4 and
-//    its error in q, cos = 1 + t^2 p(t^2) (2.5e-9 and 6e-11); the quadrant swaps and negates.
+//    its error in q, cos = 1 + t^2 p(t^2), q and p of degree 3; the quadrant swaps and negates.
+// The polynomials are minimax fits to the functions (made again in
+// tests/test_packed_normal_fit.py): P for the relative error with P(0) given, and q, rounded to
+// fp32 from the lowest order on, the rest fitted again; p rounded at once.  Their errors: ln
+// 5.8e-9 of the result, sin 2.5e-9, cos 8.7e-9.
 // Over all 2^24 uniforms (double precision): radius within 3.5e-7 (rms 4.05e-8), cos and sin
 // within 6.1e-8, no further off than logf, sqrtf and sincospif.
 template <int kV>
@@ -173,10 +179,11 @@ __device__ __forceinline__ void box_muller_parts(const uint32_t (&xa)[2 * kV],
   }
 }
 
-// The same of one pair of words by CUDA's functions: what forms Z and bf16 weights' Omega, which
-// are few (the transform above is for the full-space pass's draws and fp32 bases).  The two
-// differ in the last place, and bf16 weights at a rounding boundary show it: up to rel 1.3e-5
-// of a 1 M-weight set after a step.
+// The same of one pair of words by CUDA's functions: what forms Z, and Omega but for the panels
+// of fp32 weights at r = 4 and 8 with 4 r rows or more that clusters hold in registers
+// (zo_cholqr_small.cu; those and the full-space pass take the transform above).  The two differ in the last
+// place, and bf16 weights at a rounding boundary show it: up to rel 1.3e-5 of a 1 M-weight set
+// after a step.
 __device__ __forceinline__ float2 box_muller(uint32_t xa, uint32_t xb) {
   const float rad = sqrtf(-2.0f * logf(u01(xa)));
   float s, c;
