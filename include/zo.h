@@ -26,6 +26,12 @@
  *   leaves all buffers untouched.
  * - A context belongs to the device that was current at zo_create; each call on it
  *   makes that device current for its duration and restores the caller's device.
+ * - A caller's kernel that is launched after a call as a programmatic dependent
+ *   (cudaLaunchAttributeProgrammaticStreamSerialization) may start while the call's last
+ *   kernel is running.  Before its griddepcontrol.wait (cudaGridDependencySynchronize) it
+ *   must read none of the buffers that the call writes (W, U, V, M, Vm, gamma, Y), not even
+ *   to prefetch weights, and write none that the call reads.  Ordinary launches, copies
+ *   and events are ordered after the call as usual.
  * - Kernels that detect a problem at run time (an mbarrier wait that ran out of
  *   iterations, an internal bound check) write a code to a device status word;
  *   zo_sync_status() synchronises the stream and returns and clears it.
@@ -96,8 +102,9 @@ enum {
                                    else, at r in {4, 8}, the narrow-tile FMA pass when its
                                    tiles number at most half of the 32-row tiles (sets of
                                    thin matrices such as LoRA factors); else the FMA pass,
-                               1 = FMA path on full tiles (64 x 128; at r in {4, 8} and at
-                               most four waves of them one-launch passes on 32-row tiles),
+                               1 = FMA path on full tiles (64 x 128; perturbations at r in
+                               {4, 8} of sets of at most four 32-row tiles per SM by a
+                               one-launch pass on those),
                                2 = tcgen05 path,
                                3 = FMA path on narrow tiles (r in {4, 8}).  All FMA
                                tilings give bit-identical weights. */
@@ -106,21 +113,23 @@ enum {
                                      CTA first waits on a barrier nothing arrives on, so its
                                      bounded wait (~0.1 s) runs out; that pass then reports
                                      ZO_ERR_TIMEOUT via zo_sync_status and leaves W partly
-                                     updated.  If an SM-pair or few-token zo_linear_perturbed
-                                     call comes first, it takes the hook instead: its Y tiles wait for
-                                     S rows that are never counted as written, give up after
+                                     updated.  If an SM-pair or few-token
+                                     zo_linear_perturbed call comes first, it takes the
+                                     hook instead: its Y tiles wait for S rows that are never counted as written, give up after
                                      ~0.1 s and leave Y partly written.  Nothing faults; the
                                      context stays usable. */
   ZO_OPTION_LINEAR_TILE = 3, /* tiles (rows of X x columns of Y) of zo_linear_perturbed's
                                Y = X W^T + S U^T GEMM: 0 = automatic (up to 128 tokens at
-                               r <= 64 all of them x a few columns of Y per CTA, tiling 9; else
+                               r <= 64, where one wave of CTAs covers Y, all of them x a few
+                               columns of Y per CTA, which zo_linear_tiling reports as 9; else
                                the SM-pair tiling whose busiest pair has the least operand
                                traffic; the single-CTA ones if no 2-CTA cluster fits),
                                1 = 128 x 256,
                                2 = 256 x 256, 3 = 256 x 224 on single CTAs (S = X P^T by a
                                separate split-K kernel), 4 .. 8 = 256 x 256, 240, 224, 192,
                                128 on SM pairs (M = 256 MMAs across a 2-CTA cluster, S in
-                               the same launch).  The tilings of one family give
+                               the same launch).  9 cannot be set.  The tilings of one
+                               family, 9 and 4 .. 8 together, give
                                bit-identical Y; the two families may differ in the last
                                bits of S (each splits S's K in ranges of its own).  At
                                r in {64, 128} only the SM-pair tilings exist: a call with
@@ -171,10 +180,12 @@ ZO_API zo_status zo_destroy(zo_ctx* ctx);
  * and Omega_V (n x r, tag 3) from the counter contract and writes into U_i and V_i
  * the Q of their thin QR factorisation with diag(R) > 0, i.e. Q with column c
  * multiplied by sgn(R_cc) (Eq. (11), sgn(0) = +1).  That factor is unique; panels
- * with at least 4r rows at r >= 16 (and tall ones of fp32 weights at r = 4 and 8)
- * reach it by CholeskyQR2 (two rounds of Cholesky
- * of the Gram matrix and a triangular solve), the others by a batched Householder
- * TSQR with the sign fix.  A Gram matrix without a positive pivot (not expected for
+ * with at least 4r rows at r >= 16, and of fp32 weights those with 4r to 40960 rows at
+ * r = 4 and 4r to 16384 at r = 8, reach it by CholeskyQR2 (two rounds of Cholesky of the
+ * Gram matrix and a triangular solve), the others by Householder reflections with the
+ * sign fix (a batched TSQR, or one warp for a short panel).  A panel's bits depend on the
+ * seed, j, its index and its size, not on the other matrices of the context; at r = 4 and 8
+ * bases of fp32 and of bf16 weights of one index may differ in the last places.  A Gram matrix without a positive pivot (not expected for
  * such panels) makes the next zo_sync_status return ZO_ERR_CUDA.  reset_moments != 0
  * also zeroes M_i and Vm_i.
  */
@@ -282,8 +293,9 @@ ZO_API zo_status zo_get_timing(zo_ctx* ctx, double* total_ms, int64_t* launches)
    (1 = FMA on full tiles, 2 = tcgen05, 3 = FMA on narrow tiles). */
 ZO_API int32_t zo_wpass_path(const zo_ctx* ctx);
 
-/* zo_linear_tiling -- the tiling (1 .. 8, as ZO_OPTION_LINEAR_TILE) of the Y GEMM that
- * the last zo_linear_perturbed launched; 0 before the first call or for a null ctx. */
+/* zo_linear_tiling -- the tiling of the Y GEMM that the last zo_linear_perturbed launched:
+ * 1 .. 8 as ZO_OPTION_LINEAR_TILE, or 9, the few-token kernel, which the automatic choice
+ * takes and the option cannot name; 0 before the first call or for a null ctx. */
 ZO_API int32_t zo_linear_tiling(const zo_ctx* ctx);
 
 /* zo_kernel_launches -- number of kernels this context has launched since zo_create. */
@@ -299,9 +311,12 @@ ZO_API zo_status zo_philox_fill(uint64_t seed, uint32_t x1, uint32_t x2, uint32_
 
 /*
  * zo_normal_fill -- the Gaussian stream of the contract (uniform + Box-Muller on
- * lane pairs), elements 0..n-1, fp32, into device memory.  This is exactly how
- * Z_i^(k) (x1 = i, x2 = t, x3 = 1 << 24 | k) and Omega (x2 = j, x3 = tag << 24)
- * are drawn inside the other calls.
+ * lane pairs), elements 0..n-1, fp32, into device memory.  Z_i^(k) (x1 = i, x2 = t,
+ * x3 = 1 << 24 | k) and Omega (x2 = j, x3 = tag << 24) have exactly these bits inside the
+ * other calls, with one exception: at r = 4 and 8 Omega of fp32 weights' panels that
+ * zo_refresh takes by CholeskyQR2 is formed from the same uniforms by another fp32
+ * evaluation of the transform, as zo_mezo_perturb's normals are.  Either evaluation is
+ * within 2e-6 of the exact normals.
  */
 ZO_API zo_status zo_normal_fill(uint64_t seed, uint32_t x1, uint32_t x2, uint32_t x3, float* out,
                          int64_t n, void* stream);
