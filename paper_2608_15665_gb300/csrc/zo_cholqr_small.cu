@@ -1,5 +1,5 @@
-// Subspace refresh of fp32 weights at r = 4 and 8: Alg. 1's Haar factor of every panel in one launch, the
-// panel held in registers.
+// Subspace refresh of fp32 weights at r = 4 and 8: Alg. 1's Haar factor of every panel in one
+// launch, the panel held in registers.
 //
 // Tall panels (rows >= 4 r, at most 8 CTAs' worth) by CholeskyQR2 as in zo_cholqr.cu -- the
 // unique Q with diag(R) > 0 of Eq. (11), twice Q <- X L^-T with L L^T = X^T X -- by one
@@ -25,6 +25,19 @@ namespace {
 constexpr int kThreads = 256;
 constexpr int kWarps = kThreads / 32;
 
+// Rows per thread: about the most that 128 registers (two CTAs per SM) hold, because a panel that
+// fits fewer CTAs needs fewer exchanges, and one that fits no cluster falls back to the TSQR.  At
+// r = 4 20 rows spill 32 bytes, 22 564; at r = 8 8 rows spill none, 10 96 and 12 232.  A refresh of
+// 160 fp32 matrices 8 x L in us (one 8 x 8192 matrix alone 16.6 with 20 rows, 14.4 with 10):
+//   r = 4, L =   1024   4096   5120   8192  11008  16384  20480  32768  40960
+//     10 rows     8.3   22.6   22.6   30.8   45.1   51.2   55.4    163    201
+//     16 rows    10.3   16.5   24.7   29.0   37.5   43.1   60.5     75    201
+//     20 rows    10.3   16.5   18.5   30.8   39.9   45.8   51.4     84     95
+//     22 rows    10.3   18.5   20.6   32.8   36.9   47.9   53.9     88     98
+//   r = 8
+//      4 rows    12.4   41.2   59.7   66.8    164    195    236    356    433
+//      8 rows    14.9   39.0   47.9   55.8     85     97    238    356    433
+//     10 rows    16.7   41.0   43.1   58.8     92    103    113    356    433
 template <int R>
 struct SmallShape {
   static constexpr int kRPT = R == 4 ? 20 : 8;             // rows per thread

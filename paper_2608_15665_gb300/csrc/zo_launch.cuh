@@ -5,7 +5,8 @@
 // that earlier work in the stream may touch (constant tables of the context aside), in every
 // CTA, and pdl_trigger() after it, which lets the stream's next such launch be scheduled once
 // every CTA of this grid is running: a waiting grid can therefore not keep this one's CTAs
-// from an SM.  As each of these grids waits for its predecessor before it does anything, its
+// from an SM.  A pass that triggers still writes W after it: whoever launches a dependent behind
+// it waits before reading W, as these kernels do.  As each of these grids waits for its predecessor before it does anything, its
 // completion implies that of all earlier work.  The long tensor-core weight passes do not
 // trigger: the next pass's coefficient kernel, resident beside them from their start, cost
 // the 7B set's r = 32 pass 4% (4.16 ms against 3.99).

@@ -26,7 +26,12 @@
 // row for 64 elements of K, or HBM's 2 bytes per weight take longer (12288 x 12288: 49 us at
 // one token, 6.2 TB/s).  Measured at 1, 97 and 128 tokens, r = 32, against the SM-pair kernel's
 // best tiling: 4096 x 4096 17.6, 17.3, 17.3 us (28, 26, 26); 11008 x 4096 19.4, 20.2, 22.5 us
-// (41, 28, 29); 4096 x 11008 35, 37, 37 us (55, 54, 54).  Splitting K over a cluster of CTAs
+// (41, 28, 29); 4096 x 11008 35, 37, 37 us (55, 54, 54).  Over 13 shapes from 264 x 136 to 12288 x
+// 768 and 768 x 12288, r = 16, 32 and 64 and 1 to 128 tokens it takes 0.41 to 0.80 of that kernel's
+// time, least ahead on tall W at 128 tokens.  Short K at 1, 32, 128 tokens: 512 x 512 at r = 16 6.6,
+// 6.7, 7.1 us (10.4, 10.6, 11.3), at r = 64 6.9, 7.0, 7.5 (11.0, 11.3, 11.7); 4096 x 512 at r = 16
+// 7.2, 7.4, 8.0 (10.9, 11.2, 11.5), at r = 64 7.9, 8.1, 8.8 (12.6, 12.5, 13.2); 16384 x 512 at r = 32
+// 8.9, 9.4, 9.8 (12.0, 12.1, 12.6).  Splitting K over a cluster of CTAs
 // cuts the chain (4096 x 11008: 19 us at one token) but sums in another order, and its exchange
 // grows with the tokens (25 us at 97).
 //

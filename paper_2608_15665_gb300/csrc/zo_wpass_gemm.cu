@@ -18,8 +18,9 @@
 //    r = 32 and 64 that makes 64-row tiles faster than 128-row ones with two CTAs (164 and
 //    267 us against 176 and 295), elsewhere they are within 3%; 32-row tiles are slower
 //    (217 and 385 us).  At r <= 16, where there is little arithmetic to hide W's latency under,
-//    four CTAs, at 64 registers: 121 -> 115 us at r = 16, 112 -> 105 at r = 8 (bf16: 85 -> 77);
-//    five or six spill (160 and 245 us at r = 8).  From r = 32 on, fewer, 8 x 8 register tiles
+//    four CTAs, at 64 registers, although r = 16 then spills (32 bytes stored, 76 loaded; r = 4 12
+//    and 32, r = 8 nothing): 121 -> 115 us at r = 16, 112 -> 105 at r = 8 (bf16: 85 -> 77).  Five
+//    or six spill far more (160 and 245 us at r = 8).  From r = 32 on, fewer, 8 x 8 register tiles
 //    read less from shared memory, of which the 4 x 8 ones take 67%, but leave too few warps
 //    (128 threads: 192 us at r = 32).
 #include "zo_fma_common.cuh"
