@@ -17,6 +17,7 @@
 
 #include "zo_cluster.cuh"
 #include "zo_kernels.h"
+#include "zo_launch.cuh"
 #include "zo_reduce.cuh"
 
 namespace zo {
@@ -237,21 +238,10 @@ template <int R>
 cudaError_t launch_small_r(const CqPanel* tall, int n_tall, const CqPanel* shorts, int n_short,
                            int ctas, uint64_t seed, uint32_t refresh_idx, uint32_t* d_status,
                            cudaStream_t s) {
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(n_tall * ctas + (n_short + kWarps - 1) / kWarps, 1, 1);
-  cfg.blockDim = dim3(kThreads, 1, 1);
-  cfg.stream = s;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = ctas;
-  attr[0].val.clusterDim.y = 1;
-  attr[0].val.clusterDim.z = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = ctas > 1 ? 1 : 0;
-  cudaError_t e = cudaLaunchKernelEx(&cfg, cq_small_kernel<R>, tall, n_tall, shorts, n_short, ctas,
-                                     seed, refresh_idx, d_status);
-  if (e != cudaSuccess) return e;
-  return cudaGetLastError();
+  const unsigned grid = (unsigned)(n_tall * ctas + (n_short + kWarps - 1) / kWarps);
+  return launch_dependent(cq_small_kernel<R>, grid, kThreads, 0, s, (unsigned)ctas,
+                          /*dependent=*/false, tall, n_tall, shorts, n_short, ctas, seed, refresh_idx,
+                          d_status);
 }
 
 }  // namespace

@@ -44,6 +44,7 @@
 #include <cuda.h>
 
 #include "zo_kernels.h"
+#include "zo_launch.cuh"
 #include "zo_linear_common.cuh"
 #include "zo_sm100.cuh"
 #include "zo_tc_common.cuh"
@@ -142,8 +143,8 @@ linear_few_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
   const uint32_t tmem = sh.tmem_base;
   // a programmatic dependent of the stream's previous kernel: everything below may touch
   // memory that kernel writes
-  asm volatile("griddepcontrol.wait;" ::: "memory");
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  pdl_wait();
+  pdl_trigger();
   const volatile int* abort = &sh.abort_flag;
 
   if (warp == 0 && lane == 0) {
@@ -310,19 +311,8 @@ cudaError_t launch_few_r(const CUtensorMap& tm_x, const CUtensorMap& tm_xs, cons
   cudaError_t e = cudaFuncSetAttribute(linear_few_kernel<R>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(ctas, 1, 1);
-  cfg.blockDim = dim3(kThreads, 1, 1);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = s;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  e = cudaLaunchKernelEx(&cfg, linear_few_kernel<R>, tm_x, tm_xs, tm_w, tm_pk, tm_s, tm_u, args);
-  if (e != cudaSuccess) return e;
-  return cudaGetLastError();
+  return launch_dependent(linear_few_kernel<R>, (unsigned)ctas, kThreads, smem, s, 1, true, tm_x, tm_xs,
+                          tm_w, tm_pk, tm_s, tm_u, args);
 }
 
 int64_t ceil_div(int64_t a, int64_t b) { return (a + b - 1) / b; }

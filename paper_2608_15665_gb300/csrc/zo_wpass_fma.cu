@@ -270,11 +270,9 @@ __device__ __forceinline__ void narrow_tile(const MatDesc& md, const NarrowMat& 
     const float* U0 = md.U + row0 * R;
     for (int idx = tid; idx < rows * (R / 4); idx += kNarrowThreads) {
       const bool live = idx < row_end * (R / 4);
-      const uint32_t dst = (uint32_t)__cvta_generic_to_shared(Us + 4 * idx);
-      asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(dst),
-                   "l"(live ? U0 + 4 * idx : U0), "r"(live ? 16 : 0) : "memory");
+      cp_async_16(Us + 4 * idx, live ? U0 + 4 * idx : U0, live ? 16 : 0);
     }
-    asm volatile("cp.async.commit_group;\n" ::: "memory");
+    cp_async_commit();
   }
   // V rows of the P columns this thread forms
   const int col_end = (int)min64(cols, md.n - col0);     // live columns of the tile
@@ -306,7 +304,7 @@ __device__ __forceinline__ void narrow_tile(const MatDesc& md, const NarrowMat& 
         wraw[j] = *reinterpret_cast<const uint4*>(Wt + (int64_t)rl * md.ldw + cl * VEC);
     }
   }
-  asm volatile("cp.async.wait_all;\n" ::: "memory");
+  cp_async_wait<0>();
   __syncthreads();
 
   // P[k][c] = sum_b C[k][b] V[col0 + c][b] for the tile's columns (zero past n)
